@@ -1,11 +1,12 @@
 // Sparse-times-dense products of Algorithm 1 (A1 F, A2 Y) and Algorithm 2
 // (A2^T Y, A1^T F') of the paper, in gather form: every output row is owned by
-// one warp, so no atomics are used and results are deterministic.
+// one group of lanes, so no atomics are used and results are deterministic.
 //
 // y[b][r][n] = sum_{e in row r} A[e] * x[b][col[e]][n],  n < ncols.
-// Lanes own consecutive dense columns (float4 when rows are 16-byte aligned);
-// a row's (column, value) pairs are loaded 32 at a time and broadcast with
-// warp shuffles.  Entries are FP32 or BF16; accumulation is FP32.
+// A group of lanes owns a row and its lanes consecutive dense columns, as
+// many rows to a warp as the width leaves room for; a row's (column, value)
+// pairs are loaded coalesced, staged in shared memory and read back one by
+// one.  Entries are FP32 or BF16; accumulation is FP32.
 //
 // A1 by rotation (SrtRot): with n_phi a multiple of 4, sensor column
 // j + n_phi/4 sees the image turned by 90 degrees about the axis, so
@@ -16,13 +17,12 @@
 // rot^s(p).  Mode 2 (A1^T): output row p walks, for s = 0..3, stored row
 // rot^-s(p) of the stored transpose and gathers row (j + s n_phi/4, l): the
 // same terms in the same order (ascending j, then l) as the full transpose.
-#include <type_traits>
-
 #include "common.cuh"
 
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int kSMs = 152;
 #ifdef SRT_CHECKS
 __device__ unsigned long long g_viol;  // gathered rows outside their operand
 #endif
@@ -58,21 +58,21 @@ __device__ __forceinline__ int rot_pixel(int p, int s, int ms, uint64_t magic, b
 }
 
 // Block-to-rows order.  Rows come in G groups of R rows (r = g*R + i).  With
-// G > 0 a block owns a tile of TG groups x 8/TG consecutive i, and
+// G > 0 a block owns a tile of TG groups x RPB/TG consecutive i, and
 // consecutive blocks take the same chunk of i in consecutive group tiles
 // (chunk-major): all groups advance through i together, so the dense rows
 // gathered by concurrently running blocks stay within a narrow band of the
-// operand (L2 reuse), while a block's 8 warps gather overlapping rows (L1
+// operand (L2 reuse), while a block's rows gather overlapping rows (L1
 // reuse).  With G = 0 blocks take consecutive rows.  With S > 0 the G x R
 // grid is walked in S x S super-tiles (S dividing G and R), tiles row-major
 // inside each: the dense rows gathered by concurrently running blocks then
 // belong to a compact patch instead of a band across all G groups (A1^T:
 // pixels, whose circles through a 64 x 64 patch cover ~40% of the operand
-// instead of most of it).
-__device__ __forceinline__ int block_row(int G, int R, int TG, int S) {
-  const int w = threadIdx.x >> 5;
-  if (G <= 0) return blockIdx.x * (blockDim.x >> 5) + w;
-  const int TI = 8 / TG;
+// instead of most of it).  w: this row's place among the block's RPB rows.
+template <int RPB>
+__device__ __forceinline__ int block_row(int G, int R, int TG, int S, int w) {
+  if (G <= 0) return blockIdx.x * RPB + w;
+  const int TI = RPB / TG;
   if (S > 0) {
     const int per_row = S / TG, bpt = per_row * (S / TI);
     const int st = blockIdx.x / bpt, r = blockIdx.x - st * bpt;
@@ -96,130 +96,83 @@ struct Rows {
   SrtRot rot;
   uint64_t magic;  // ceil(2^40 / rot.ms)
   int xrows;       // rows of the gathered operand (debug-build checks)
-  int64_t ldn;     // > 0: reshape P1 fused (k_spmm_rot), stride of Y1''s rows
-  int pack16;      // BF16 entries of A1 by rotation, pixels < 2^16 (k_spmm_rot PK)
+  int64_t ldn;     // > 0: reshape P1 fused, stride of Y1''s rows
 };
 
-// Stored row and gathered-row remap of segment s of output row `row`.
-// Mode 1, the 8-fold form: is output column j served by a mirrored column?
-__device__ __forceinline__ bool seg_mirrored(const Rows& A, int j) {
-  return A.rot.mirror && 2 * (j % A.rot.q) > A.rot.q;
-}
-template <int MODE>
-__device__ __forceinline__ int seg_row(const Rows& A, int row, int s) {
-  if (MODE == 1) {
-    const int j = row / A.rot.n_ell, l = row - j * A.rot.n_ell;
-    const int js = j % A.rot.q;
-    return (seg_mirrored(A, j) ? A.rot.q - js : js) * A.rot.n_ell + l;
-  }
-  if (MODE == 2) return rot_pixel(row, 4 - s, A.rot.ms, A.magic);
-  return row;
-}
-// Gathered row of stored column c in segment s (t: quarter turns of the row,
-// mir: mirrored first).
-template <int MODE>
-__device__ __forceinline__ int seg_col(const Rows& A, int t, bool mir, int s, int c) {
-  if (MODE == 1) return rot_pixel(c, t, A.rot.ms, A.magic, mir);
-  if (MODE == 2) return c + s * A.rot.q * A.rot.n_ell;
-  return c;
-}
-
-// Rows stored as they are (no rotation).  rowptr is the launch's first row's
-// pointer.  (A single kernel for both cases, with the row bookkeeping behind
-// a struct passed by reference, measured 3% slower.)
-template <typename V, int CH>
-__global__ void __launch_bounds__(256) k_spmm_plain(int rows, const int32_t* __restrict__ rowptr,
-                                                    const int32_t* __restrict__ col,
-                                                    const V* __restrict__ val,
-                                                    const float* __restrict__ x, int64_t ldx,
-                                                    int64_t bsx, float* __restrict__ y,
-                                                    int64_t ldy, int64_t bsy, int ncols, int G,
-                                                    int R, int TG, int S, int xrows) {
-  const int lane = threadIdx.x & 31;
-  const int row = block_row(G, R, TG, S);
-  if (row < 0 || row >= rows) return;
-  x += blockIdx.z * bsx;
-  y += blockIdx.z * bsy;
-  const int n0 = blockIdx.y * (128 * CH) + lane * 4;
-  float4 acc[CH];
-#pragma unroll
-  for (int q = 0; q < CH; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int e0 = rowptr[row], e1 = rowptr[row + 1];
-  for (int eb = e0; eb < e1; eb += 32) {
-    int c = 0;
-    float v = 0.f;
-    if (eb + lane < e1) {
-      c = col[eb + lane];
-      SRT_CHECK_GATHER(0, c, xrows, g_viol);
-      v = wval<V>(val[eb + lane]);
-    }
-    const int cnt = min(32, e1 - eb);
-    // not unrolled: 31 registers, 64 resident warps per SM.  The products
-    // wait on their gathers, and more warps in flight beat the deeper
-    // per-warp schedule of an unrolled loop (40 registers, 48 warps): 4.5%
-    // faster, same summation order.
-#pragma unroll 1
-    for (int i = 0; i < cnt; ++i) {
-      const int ci = __shfl_sync(FULL, c, i);
-      const float vi = __shfl_sync(FULL, v, i);
-      const float* xr = x + (int64_t)ci * ldx;
-#pragma unroll
-      for (int q = 0; q < CH; ++q) {
-        const int n = n0 + q * 128;
-        if (n < ncols) {
-          const float4 xv = srt_ldg_keep(xr + n);
-          acc[q].x = fmaf(vi, xv.x, acc[q].x);
-          acc[q].y = fmaf(vi, xv.y, acc[q].y);
-          acc[q].z = fmaf(vi, xv.z, acc[q].z);
-          acc[q].w = fmaf(vi, xv.w, acc[q].w);
-        }
-      }
-    }
-  }
-  float* yr = y + (int64_t)row * ldy;
-#pragma unroll
-  for (int q = 0; q < CH; ++q) {
-    const int n = n0 + q * 128;
-    if (n < ncols) *reinterpret_cast<float4*>(yr + n) = acc[q];
+// VW consecutive dense columns of a gathered row.
+template <int VW>
+__device__ __forceinline__ void ld_cols(const float* p, float (&v)[VW]) {
+  if constexpr (VW == 4) {
+    const float4 q = srt_ldg_keep(p);
+    v[0] = q.x;
+    v[1] = q.y;
+    v[2] = q.z;
+    v[3] = q.w;
+  } else if constexpr (VW == 2) {
+    const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+    v[0] = q.x;
+    v[1] = q.y;
+  } else {
+    v[0] = __ldg(p);
   }
 }
 
-// A1 / A1^T from the stored quarter of A1 (the plain loop with the stored
-// row and the gathered row remapped; scalar parameters only).  MODE 1: row
-// (j, l) of A1 from stored row (j mod q, l), pixels turned j / q times.
-// MODE 2: row p of A1^T from stored rows rot^-s(p), s = 0..3, gathered rows
-// shifted by s q n_ell.  rowptr: the stored matrix's own pointers.
-// TR (MODE 1, blocks of 4 sensor columns x 2 radii, G = n_phi, R = n_ell):
-// the reshape P1 in the epilogue.  The block's 8 rows go through shared
-// memory, 128 slabs at a time, and are written as Y1'[(l, k)][b G + j],
-// row stride ldn, 16 bytes (4 sensor columns) per radius and slab.
-// PK (BF16 entries, MODE 1, fewer than 2^16 pixels): each lane packs its
-// entry's turned pixel and BF16 value into one word, so the warp broadcasts
-// an entry with one shuffle instead of two (same pixel, same value; the
-// shuffles share the L1 data pipe with the gathers: A1 1.580 -> 1.506 ms
-// at 256^3 with BF16 entries).
-template <typename V, int CH, int MODE, bool TR, bool PK>
-__global__ void __launch_bounds__(256) k_spmm_rot(int rows, int r0,
-                                                  const int32_t* __restrict__ rowptr,
-                                                  const int32_t* __restrict__ col,
-                                                  const V* __restrict__ val,
-                                                  const float* __restrict__ x, int64_t ldx,
-                                                  int64_t bsx, float* __restrict__ y, int64_t ldy,
-                                                  int64_t bsy, int ncols, int G, int R, int TG,
-                                                  int S, int ms, int n_ell, int q,
-                                                  int mirror, uint64_t magic, int xrows,
-                                                  int64_t ldn) {
-  const int lane = threadIdx.x & 31;
-  const int lr = block_row(G, R, TG, S);
+// A group of GL lanes owns an output row, 32 / GL rows to a warp; a lane
+// owns VW consecutive columns of each of CH chunks of VW GL columns.  The
+// row's entries are loaded EB at a time by the group's lanes, the gathered
+// row remapped there (MODE 1: A1 row (j, l) from stored row (j mod q, l),
+// pixels turned j / q times, mirrored first where the stored column is a
+// mirror image; MODE 2: A1^T row p from stored rows rot^-s(p), s = 0..3,
+// gathered rows shifted by s q n_ell), and put in shared memory as (row,
+// value) pairs that the group then reads back.
+//
+// What bounds it.  A gathered operand feeds one FMA, so the L1 data pipe
+// (128 B a cycle per SM) is the limit at full width: 93% busy at 256^3,
+// where each entry takes 8 cycles for its 1 KB and 2 for broadcasting row
+// and value by two shuffles.  The pair read back by one 8-byte shared load
+// takes 1 (a load that all lanes read from one shared address costs half of
+// what it writes to registers): A1 at 256^3 1.578 -> 1.526 ms.  Below 128
+// columns a whole warp to a row leaves lanes idle and spends the same loop
+// on fewer columns; with GL lanes to a row (measured, one box, FP32 entries,
+// a warp to a row before): 8 x 64^3 446 -> 224 us, 128^3 416 -> 346, 192^3
+// 1180 -> 1089.  U gathers are requested before their FMAs: two cost no
+// registers' worth of residency (32, 64 warps per SM) and gain 4% at 128^3;
+// four cost 6% at 256^3 but win where the launch cannot fill the GPU.
+// A row's entries are summed in the same order in every variant.
+//
+// TR (MODE 1, GL = 32, blocks of 4 sensor columns x 2 radii, G = n_phi, R =
+// n_ell): the reshape P1 in the epilogue.  The block's 8 rows go through
+// shared memory, 128 slabs at a time, and are written as Y1'[(l, k)][b G +
+// j], row stride ldn, 16 bytes (4 sensor columns) per radius and slab.
+template <typename V, int VW, int CH, int GL, int MODE, bool TR, int U>
+__global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* __restrict__ rowptr,
+                                              const int32_t* __restrict__ col,
+                                              const V* __restrict__ val,
+                                              const float* __restrict__ x, int64_t ldx,
+                                              int64_t bsx, float* __restrict__ y, int64_t ldy,
+                                              int64_t bsy, int ncols, int G, int R, int TG, int S,
+                                              int ms, int n_ell, int q, int mirror,
+                                              uint64_t magic, int xrows, int64_t ldn) {
+  constexpr int NR = 32 / GL, EB = GL == 32 ? 32 : 16;
+  // 384 or 512 columns to a warp: the pairs stay in registers and go round
+  // by shuffles, whose share of the row's time is small there, and the
+  // shared loads' extra registers cost more (A2 as CSR at 3072 columns 244
+  // us, 268 through shared memory; A2^T 249, 316)
+  constexpr bool SH = GL == 32 && VW == 4 && CH > 2;
+  __shared__ int2 stage[SH ? 1 : 8][NR][EB + (NR > 1 ? 1 : 0)];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane / GL, sl = lane % GL;
+  const int lr = block_row<8 * NR>(G, R, TG, S, w * NR + sub);
   const bool mine = lr >= 0 && lr < rows;
-  if (!TR && !mine) return;  // (TR: every warp reaches the block barrier)
+  if (!TR && NR == 1 && !mine) return;  // (otherwise every lane reaches the barriers)
   const int row = r0 + (mine ? lr : 0);
   x += blockIdx.z * bsx;
   if (!TR) y += blockIdx.z * bsy;
-  const int n0 = blockIdx.y * (128 * CH) + lane * 4;
-  float4 acc[CH];
+  const int n0 = blockIdx.y * (VW * GL * CH) + sl * VW;
+  float acc[CH][VW];
 #pragma unroll
-  for (int k = 0; k < CH; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = 0; k < CH; ++k)
+#pragma unroll
+    for (int i = 0; i < VW; ++i) acc[k][i] = 0.f;
   int t = 0, sr = row;
   bool mir = false;
   if (MODE == 1) {
@@ -232,194 +185,234 @@ __global__ void __launch_bounds__(256) k_spmm_rot(int rows, int r0,
     }
     sr = js * n_ell + l;
   }
+  int2* st = stage[SH ? 0 : w][sub];
 #pragma unroll 1
   for (int s = 0; s < (MODE == 2 ? 4 : 1); ++s) {
     if (MODE == 2) sr = rot_pixel(row, 4 - s, ms, magic);
     const int off = MODE == 2 ? s * q * n_ell : 0;
-    const int e0 = rowptr[sr], e1 = TR && !mine ? e0 : rowptr[sr + 1];
-    for (int eb = e0; eb < e1; eb += 32) {
-      int c = 0;
-      float v = 0.f;
-      uint32_t pw = 0;
-      if (eb + lane < e1) {
-        c = col[eb + lane];
-        c = MODE == 1 ? rot_pixel(c, t, ms, magic, mir) : c + off;
-        SRT_CHECK_GATHER(0, c, xrows, g_viol);
-        if constexpr (PK)
-          pw = ((uint32_t)c << 16) | (uint32_t)val[eb + lane];
-        else
-          v = wval<V>(val[eb + lane]);
-      }
-      const int cnt = min(32, e1 - eb);
+    const int e0 = rowptr[sr], e1 = mine ? rowptr[sr + 1] : e0;
+    // batches run in step over the warp's rows (an exhausted row idles)
+    const int len = NR > 1 ? (int)__reduce_max_sync(FULL, (unsigned)(e1 - e0)) : e1 - e0;
 #pragma unroll 1
-      for (int i = 0; i < cnt; ++i) {  // not unrolled, as in k_spmm_plain
-        int ci;
-        float vi;
-        if constexpr (PK) {
-          const uint32_t wi = __shfl_sync(FULL, pw, i);
-          ci = (int)(wi >> 16);
-          vi = __uint_as_float(wi << 16);
-        } else {
-          ci = __shfl_sync(FULL, c, i);
-          vi = __shfl_sync(FULL, v, i);
+    for (int b = 0; b < len; b += EB) {
+      const int eb = e0 + b;
+      if constexpr (SH) {
+        int c = 0;
+        float v = 0.f;
+        if (eb + lane < e1) {
+          c = col[eb + lane];
+          if (MODE == 1) c = rot_pixel(c, t, ms, magic, mir);
+          if (MODE == 2) c += off;
+          SRT_CHECK_GATHER(0, c, xrows, g_viol);
+          v = wval<V>(val[eb + lane]);
         }
-        const float* xr = x + (int64_t)ci * ldx;
+        const int cnt = min(32, e1 - eb);
+#pragma unroll 1
+        for (int i = 0; i < cnt; ++i) {
+          const int ci = __shfl_sync(FULL, c, i);
+          const float vi = __shfl_sync(FULL, v, i);
+          const float* xr = x + (int64_t)ci * ldx;
+#pragma unroll
+          for (int k = 0; k < CH; ++k) {
+            const int n = n0 + k * (VW * GL);
+            if (n < ncols) {
+              float xv[VW];
+              ld_cols<VW>(xr + n, xv);
+#pragma unroll
+              for (int u = 0; u < VW; ++u) acc[k][u] = fmaf(vi, xv[u], acc[k][u]);
+            }
+          }
+        }
+        continue;
+      }
+#pragma unroll
+      for (int i = sl; i < EB; i += GL) {
+        if (eb + i < e1) {
+          int c = col[eb + i];
+          if (MODE == 1) c = rot_pixel(c, t, ms, magic, mir);
+          if (MODE == 2) c += off;
+          SRT_CHECK_GATHER(0, c, xrows, g_viol);
+          st[i] = make_int2(c, __float_as_int(wval<V>(val[eb + i])));
+        }
+      }
+      __syncwarp();
+      const int cnt = min(EB, e1 - eb);
+      int i = 0;
+#pragma unroll 1
+      for (; i + U <= cnt; i += U) {
+        float xv[U][CH][VW], vi[U];
+#pragma unroll
+        for (int h = 0; h < U; ++h) {
+          const int2 en = st[i + h];
+          vi[h] = __int_as_float(en.y);
+          const float* xr = x + (int64_t)en.x * ldx;
+#pragma unroll
+          for (int k = 0; k < CH; ++k)
+            if (n0 + k * (VW * GL) < ncols) ld_cols<VW>(xr + n0 + k * (VW * GL), xv[h][k]);
+        }
+#pragma unroll
+        for (int h = 0; h < U; ++h)
+#pragma unroll
+          for (int k = 0; k < CH; ++k)
+            if (n0 + k * (VW * GL) < ncols) {
+#pragma unroll
+              for (int u = 0; u < VW; ++u) acc[k][u] = fmaf(vi[h], xv[h][k][u], acc[k][u]);
+            }
+      }
+#pragma unroll 1
+      for (; i < cnt; ++i) {
+        const int2 en = st[i];
+        const float vi = __int_as_float(en.y);
+        const float* xr = x + (int64_t)en.x * ldx;
 #pragma unroll
         for (int k = 0; k < CH; ++k) {
-          const int n = n0 + k * 128;
+          const int n = n0 + k * (VW * GL);
           if (n < ncols) {
-            const float4 xv = srt_ldg_keep(xr + n);
-            acc[k].x = fmaf(vi, xv.x, acc[k].x);
-            acc[k].y = fmaf(vi, xv.y, acc[k].y);
-            acc[k].z = fmaf(vi, xv.z, acc[k].z);
-            acc[k].w = fmaf(vi, xv.w, acc[k].w);
+            float xv[VW];
+            ld_cols<VW>(xr + n, xv);
+#pragma unroll
+            for (int u = 0; u < VW; ++u) acc[k][u] = fmaf(vi, xv[u], acc[k][u]);
           }
         }
       }
+      __syncwarp();
     }
   }
   if (!TR) {
+    if (!mine) return;
     float* yr = y + (int64_t)lr * ldy;
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
-      const int n = n0 + k * 128;
-      if (n < ncols) *reinterpret_cast<float4*>(yr + n) = acc[k];
+      const int n = n0 + k * (VW * GL);
+      if (n >= ncols) continue;
+      if constexpr (VW == 4)
+        *reinterpret_cast<float4*>(yr + n) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+      else if constexpr (VW == 2)
+        *reinterpret_cast<float2*>(yr + n) = make_float2(acc[k][0], acc[k][1]);
+      else
+        yr[n] = acc[k][0];
     }
     return;
   }
   // fused P1: Sb[w][n] holds row w = 2 jl + il (column j0 + jl, radius
   // l0 + il) of the block, 128 slabs n; a thread then writes one radius and
   // slab of the 4 columns
-  __shared__ __align__(16) float Sb[8 * 128];
-  const int w = threadIdx.x >> 5, tiles = (G + 3) / 4;
-  const int c = blockIdx.x / tiles, tt = blockIdx.x - c * tiles;
-  const int il = threadIdx.x >> 7, nl = threadIdx.x & 127;
-  const int l = 2 * c + il;
-  const int64_t cb = (int64_t)blockIdx.z * G + 4 * tt;  // column b G + j0 of Y1'
+  if constexpr (TR) {
+    __shared__ __align__(16) float Sb[8 * 128];
+    const int tiles = (G + 3) / 4;
+    const int c = blockIdx.x / tiles, tt = blockIdx.x - c * tiles;
+    const int il = threadIdx.x >> 7, nl = threadIdx.x & 127;
+    const int l = 2 * c + il;
+    const int64_t cb = (int64_t)blockIdx.z * G + 4 * tt;  // column b G + j0 of Y1'
 #pragma unroll
-  for (int k = 0; k < CH; ++k) {
-    if (k) __syncthreads();  // the previous chunk's reads are done
-    *reinterpret_cast<float4*>(Sb + w * 128 + lane * 4) = acc[k];
-    __syncthreads();
-    const int n = blockIdx.y * (128 * CH) + k * 128 + nl;
-    if (l < R && n < ncols && 4 * tt < G)
-      *reinterpret_cast<float4*>(y + ((int64_t)l * ncols + n) * ldn + cb) =
-          make_float4(Sb[il * 128 + nl], Sb[(2 + il) * 128 + nl], Sb[(4 + il) * 128 + nl],
-                      Sb[(6 + il) * 128 + nl]);
+    for (int k = 0; k < CH; ++k) {
+      if (k) __syncthreads();  // the previous chunk's reads are done
+      *reinterpret_cast<float4*>(Sb + w * 128 + lane * 4) =
+          make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+      __syncthreads();
+      const int n = blockIdx.y * (128 * CH) + k * 128 + nl;
+      if (l < R && n < ncols && 4 * tt < G)
+        *reinterpret_cast<float4*>(y + ((int64_t)l * ncols + n) * ldn + cb) =
+            make_float4(Sb[il * 128 + nl], Sb[(2 + il) * 128 + nl], Sb[(4 + il) * 128 + nl],
+                        Sb[(6 + il) * 128 + nl]);
+    }
   }
 }
 
-// Scalar path for any ncols / strides: lane owns columns lane + 32 i.
-template <typename V, int PER, int MODE>
-__global__ void __launch_bounds__(256) k_spmm_scalar(Rows A, const int32_t* __restrict__ rowptr,
-                                                     const int32_t* __restrict__ col,
-                                                     const V* __restrict__ val,
-                                                     const float* __restrict__ x, int64_t ldx,
-                                                     int64_t bsx, float* __restrict__ y,
-                                                     int64_t ldy, int64_t bsy, int ncols) {
-  const int lane = threadIdx.x & 31;
-  const int lr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (lr >= A.rows) return;
-  const int row = A.r0 + lr;
-  x += blockIdx.z * bsx;
-  y += blockIdx.z * bsy;
-  const int n0 = blockIdx.y * (32 * PER) + lane;
-  float acc[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-  constexpr int NSEG = MODE == 2 ? 4 : 1;
-  const int t = MODE == 1 ? (row / A.rot.n_ell) / A.rot.q : 0;
-  const bool mir = MODE == 1 && seg_mirrored(A, row / A.rot.n_ell);
-  for (int s = 0; s < NSEG; ++s) {
-    const int sr = seg_row<MODE>(A, row, s);
-    const int e0 = rowptr[sr], e1 = rowptr[sr + 1];
-    for (int eb = e0; eb < e1; eb += 32) {
-      int c = 0;
-      float v = 0.f;
-      if (eb + lane < e1) {
-        c = seg_col<MODE>(A, t, mir, s, col[eb + lane]);
-        SRT_CHECK_GATHER(0, c, A.xrows, g_viol);
-        v = wval<V>(val[eb + lane]);
-      }
-      const int cnt = min(32, e1 - eb);
-      for (int i = 0; i < cnt; ++i) {
-        const int ci = __shfl_sync(FULL, c, i);
-        const float vi = __shfl_sync(FULL, v, i);
-        const float* xr = x + (int64_t)ci * ldx;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-          const int n = n0 + q * 32;
-          if (n < ncols) acc[q] = fmaf(vi, __ldg(xr + n), acc[q]);
-        }
-      }
-    }
+// Columns of one launch: VW GL CH per group, blockIdx.y over the groups' widths.
+template <typename V, int VW, int CH, int GL, int MODE, int U, bool TR = false>
+int launch_as(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t ldx,
+              int64_t bsx, float* y, int64_t ldy, int64_t bsy, int ncols, int batch,
+              cudaStream_t st) {
+  constexpr int RPB = 8 * (32 / GL);
+  const int TI = RPB / W.TG;
+  const int S = W.S > 0 && W.S % TI == 0 ? W.S : 0;
+  const int64_t gx = S > 0     ? (int64_t)(W.G / S) * (W.R / S) * (S / W.TG) * (S / TI)
+                     : W.G > 0 ? (int64_t)((W.G + W.TG - 1) / W.TG) * ((W.R + TI - 1) / TI)
+                               : ((int64_t)W.rows + RPB - 1) / RPB;
+  const int wide = VW * GL * CH;
+  if (gx > 0x7fffffff || (ncols + wide - 1) / wide > 65535 || batch > 65535) return SRT_ERR_ARG;
+  dim3 grid((unsigned)gx, (ncols + wide - 1) / wide, batch);
+  const SrtRot& r = W.rot;
+  k_rows<V, VW, CH, GL, MODE, TR, U><<<grid, 256, 0, st>>>(
+      W.rows, W.r0, A.rowptr, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, S, r.ms,
+      r.n_ell, r.q, r.mirror, W.magic, W.xrows, W.ldn);
+  SRT_CUDA_TRY(cudaGetLastError());
+  return SRT_OK;
+}
+
+template <typename V, int VW, int MODE, int U>
+int launch_width(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t ldx,
+                 int64_t bsx, float* y, int64_t ldy, int64_t bsy, int ncols, int batch,
+                 cudaStream_t st) {
+#define SRT_ROWS(CH, GL) \
+  return launch_as<V, VW, CH, GL, MODE, U>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st)
+  const int n = (ncols + VW - 1) / VW;  // vectors of a row
+  // wide rows stored as they are: each entry's reuse over 512 columns wins
+  // over more warps (at 1024 columns 10.6 against 11.1 ms for A2 of 256^3 as CSR)
+  if constexpr (MODE == 0 && VW == 4 && U == 1) {
+    if (n > 96) SRT_ROWS(4, 32);
+    SRT_ROWS(3, 32);
   }
-  float* yr = y + (int64_t)lr * ldy;
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int n = n0 + q * 32;
-    if (n < ncols) yr[n] = acc[q];
+  // rows wider than a part in equal parts (64 float4 vectors, 128 narrower
+  // ones: what a warp covers in two chunks or in up to four light ones);
+  // then the narrowest group that covers a part
+  constexpr int P = VW == 4 ? 64 : 128;
+  const int parts = (n + P - 1) / P, m = (n + parts - 1) / parts;
+  // Too few rows for 32 warps per SM even with a half warp to a row: the
+  // time is one row's chain of gathers, and packing more rows into a warp
+  // only lengthens it to the longest of them (A1 at 32^3, 8 vectors: 13.5 us
+  // with a half warp to a row, 17.9 with four lanes; at 64^3, 44.5 against 41.2
+  // the other way round, half warps losing).
+  if (m <= 8 && (int64_t)W.rows * batch * parts <= (int64_t)2 * 32 * kSMs) SRT_ROWS(2, 16);
+  if (m <= 8) SRT_ROWS(2, 4);
+  if (m <= 16) SRT_ROWS(2, 8);
+  if constexpr (VW == 4)
+    if (m <= 24) SRT_ROWS(3, 8);
+  if (m <= 32) SRT_ROWS(2, 16);
+  if constexpr (VW == 4)
+    if (m <= 48) SRT_ROWS(3, 16);
+  if constexpr (VW != 4) {
+    if (m > 96) SRT_ROWS(4, 32);
+    if (m > 64) SRT_ROWS(3, 32);
   }
+  SRT_ROWS(2, 32);
+#undef SRT_ROWS
 }
 
 template <typename V, int MODE>
 int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t ldx, int64_t bsx,
            float* y, int64_t ldy, int64_t bsy, int ncols, int batch, cudaStream_t st) {
-  dim3 block(256);
-  const bool vec = (ncols % 4 == 0) && (ldx % 4 == 0) && (ldy % 4 == 0) && (bsx % 4 == 0) &&
-                   (bsy % 4 == 0) && ((uintptr_t)x % 16 == 0) && ((uintptr_t)y % 16 == 0);
-  const int gx = W.S > 0   ? (W.G / W.S) * (W.R / W.S) * (W.S / W.TG) * (W.S / (8 / W.TG))
-                 : W.G > 0 ? ((W.G + W.TG - 1) / W.TG) * ((W.R + 8 / W.TG - 1) / (8 / W.TG))
-                           : (W.rows + 7) / 8;
-  if (vec && MODE == 0) {
-    const int32_t* rp = A.rowptr + W.r0;
-    const int chunks = (ncols + 127) / 128;
-    const int CH = chunks >= 4 ? 4 : chunks;
-    dim3 grid(gx, CH == 4 ? (ncols + 511) / 512 : 1, batch);
-    switch (CH) {
-      case 4: k_spmm_plain<V, 4><<<grid, block, 0, st>>>(W.rows, rp, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, W.S, W.xrows); break;
-      case 3: k_spmm_plain<V, 3><<<grid, block, 0, st>>>(W.rows, rp, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, W.S, W.xrows); break;
-      case 2: k_spmm_plain<V, 2><<<grid, block, 0, st>>>(W.rows, rp, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, W.S, W.xrows); break;
-      default: k_spmm_plain<V, 1><<<grid, block, 0, st>>>(W.rows, rp, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, W.S, W.xrows); break;
+  if constexpr (MODE == 1) {
+    if (W.ldn > 0) {
+      if (ncols > 128)
+        return launch_as<V, 4, 2, 32, 1, 1, true>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+      return launch_as<V, 4, 1, 32, 1, 1, true>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
     }
-  } else if (vec) {
-    // at most 2 chunks of 128 columns per warp, wider rows across
-    // blockIdx.y: with 512 slabs, 31 registers and 64 resident warps per SM
-    // instead of 47 and 40 made A1 13% faster (17.6 -> 15.3 ms at 512^3)
-    const int chunks = (ncols + 127) / 128;
-    const int CH = chunks >= 2 ? 2 : chunks;
-    dim3 grid(gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
-    const SrtRot& r = W.rot;
-#define SRT_ROT_LAUNCH(C, T, P)                                                                 \
-  k_spmm_rot<V, C, MODE, T, P><<<grid, block, 0, st>>>(W.rows, W.r0, A.rowptr, A.col, val, x,  \
-                                                       ldx, bsx, y, ldy, bsy, ncols, W.G, W.R,  \
-                                                       W.TG, W.S, r.ms, r.n_ell, r.q,           \
-                                                       r.mirror, W.magic, W.xrows, W.ldn)
-    constexpr bool kPk = MODE == 1 && std::is_same<V, uint16_t>::value;
-    constexpr bool kTr = MODE == 1;
-    const bool tr = kTr && W.ldn > 0, pk = kPk && W.pack16;
-    if (tr && pk) {
-      if (CH == 2) SRT_ROT_LAUNCH(2, kTr, kPk);
-      else SRT_ROT_LAUNCH(1, kTr, kPk);
-    } else if (tr) {
-      if (CH == 2) SRT_ROT_LAUNCH(2, kTr, false);
-      else SRT_ROT_LAUNCH(1, kTr, false);
-    } else if (pk) {
-      if (CH == 2) SRT_ROT_LAUNCH(2, false, kPk);
-      else SRT_ROT_LAUNCH(1, false, kPk);
-    } else if (CH == 2) {
-      SRT_ROT_LAUNCH(2, false, false);
-    } else {
-      SRT_ROT_LAUNCH(1, false, false);
-    }
-#undef SRT_ROT_LAUNCH
-  } else {
-    dim3 grid((W.rows + 7) / 8, (ncols + 127) / 128, batch);
-    k_spmm_scalar<V, 4, MODE><<<grid, block, 0, st>>>(W, A.rowptr, A.col, val, x, ldx, bsx, y,
-                                                      ldy, bsy, ncols);
   }
-  SRT_CUDA_TRY(cudaGetLastError());
-  return SRT_OK;
+  const int64_t any = ncols | ldx | ldy | bsx | bsy;
+  const uintptr_t at = (uintptr_t)x | (uintptr_t)y;
+  // Four gathers in flight per row where the rows do not keep the SMs full
+  // for more than two rounds of 64 warps (75 x 75 x 53, 18090 rows: A1 44.8
+  // -> 35.8 us, A1^T 47.1 -> 36.9; 32^3: 18.6 -> 13.5), two otherwise (96^3,
+  // 24576 warps of four rows: 207 us with four, 188 with two).
+  const int lanes = any % 4 == 0 && at % 16 == 0 ? 4 : any % 2 == 0 && at % 8 == 0 ? 2 : 1;
+  const int64_t vecs = ((int64_t)ncols + lanes - 1) / lanes;
+  const int64_t per_warp = vecs > 32 ? 1 : vecs > 16 ? 2 : 4;
+  const bool few = (int64_t)W.rows * batch / per_warp <= (int64_t)128 * kSMs &&
+                   vecs <= (lanes == 4 ? 64 : 128);
+  if constexpr (MODE == 0)
+    if (lanes == 4 && vecs > 64)
+      return launch_width<V, 4, MODE, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+#define SRT_WIDTH(VW)                                                                          \
+  return few ? launch_width<V, VW, MODE, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, \
+                                            st)                                               \
+             : launch_width<V, VW, MODE, 2>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, \
+                                            st)
+  if (lanes == 4) SRT_WIDTH(4);
+  if (lanes == 2) SRT_WIDTH(2);
+  SRT_WIDTH(1);
+#undef SRT_WIDTH
 }
 
 template <typename V>
@@ -450,7 +443,7 @@ int srt_spmm(const SrtCsr& A, int wdt, const float* x, int64_t ldx, int64_t bsx,
   }
   if (G > 0 && (int64_t)G * R != rows) G = 0;
   if (TG != 1 && TG != 2 && TG != 4 && TG != 8) TG = 1;
-  if (G <= 0 || S <= 0 || G % S || R % S || S % TG || S % (8 / TG)) S = 0;
+  if (G <= 0 || S <= 0 || G % S || R % S || S % TG) S = 0;
   // gathered operand: A's columns, or for A1^T from the stored quarter
   // (mode 2) the rows (j, l) of every sensor column
   const int64_t xr = rot.mode == 2 ? (int64_t)4 * rot.q * rot.n_ell : A.cols;
@@ -463,10 +456,7 @@ int srt_spmm(const SrtCsr& A, int wdt, const float* x, int64_t ldx, int64_t bsx,
     TG = 4;
     S = 0;
   }
-  // BF16 entries of A1 turned onto fewer than 2^16 pixels: pixel and value
-  // in one 32-bit word (one shuffle per entry)
-  const int pack16 = rot.mode == 1 && wdt == SRT_BF16 && A.cols <= 65536;
-  const Rows W{(int)rows, (int)r0, G, R, TG, S, rot, magic, srt_checked_rows(xr), ldn, pack16};
+  const Rows W{(int)rows, (int)r0, G, R, TG, S, rot, magic, srt_checked_rows(xr), ldn};
   if (wdt == SRT_BF16) return dispatch<uint16_t>(A, A.v16, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
   return dispatch<float>(A, A.v32, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
 }

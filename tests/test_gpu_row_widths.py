@@ -1,0 +1,58 @@
+"""The row products at every width class of their dispatch: vectors of 4, 2
+and 1 columns, 4 to 32 lanes to a row, one to three chunks, rows split over
+blocks, few rows (four gathers in flight) and many (two), against the FP64
+oracle on seeded samples.  The bound is that of FP32 sums of a row's entries
+(at most a few hundred), 1e-5 relative, as in the parity tests."""
+import numpy as np
+import pytest
+
+from tests.gpu_helpers import geom_pair, rel_l2, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def srt():
+    import torch
+    from paper_2402_15641_gb300 import build, srt as S
+    assert torch.cuda.is_available()
+    build.build()
+    return S
+
+
+def _sample_check(srt, orc, sz, opts, batch, n_shells, n_vox):
+    g, o = geom_pair(orc, **opts, **sz)
+    plan = srt.Plan(g)
+    rng = np.random.default_rng(61)
+    f = rng.uniform(0, 1, (batch, *g.f_shape)).astype(np.float32)
+    y = rng.standard_normal((batch, *g.p_shape)).astype(np.float32)
+    p = to_np(plan.forward(to_dev(f)))
+    a = to_np(plan.adjoint(to_dev(y)))
+    sh = np.stack([rng.integers(0, n, n_shells) for n in g.p_shape], axis=1)
+    vx = np.stack([rng.integers(0, n, n_vox) for n in g.f_shape], axis=1)
+    for b in range(batch):
+        want = orc.forward_shells(o, f[b].astype(np.float64), sh)
+        assert rel_l2(p[b][sh[:, 0], sh[:, 1], sh[:, 2]], want) <= 1e-5
+        want = orc.adjoint_voxels(o, y[b].astype(np.float64), vx)
+        assert rel_l2(a[b][vx[:, 0], vx[:, 1], vx[:, 2]], want) <= 1e-5
+
+
+@pytest.mark.parametrize("mz", [1, 2, 3, 6, 9, 16, 17, 33, 36, 52, 64, 65, 70, 100, 132, 194, 260, 264])
+@pytest.mark.parametrize("form", [dict(), dict(rowwise=True), dict(csr_only=True, rowwise=True, a1_full=True)])
+def test_few_rows(srt, orc, mz, form):
+    """Slab counts that are and are not whole vectors, below and above one
+    part of 64 vectors; 12 sensor columns (quarter turns) of batch 2."""
+    sz = dict(ms=7, mz=mz, dxy=0.4, dz=0.4 / max(1, mz // 16), radius=6.0, n_phi=12, n_zs=3, n_ell=17)
+    _sample_check(srt, orc, sz, form, 2, 120, 40)
+
+
+@pytest.mark.parametrize("mz,n_phi,n_ell,form", [(132, 64, 400, dict()), (66, 90, 480, dict()),
+                                                 (101, 64, 400, dict(a1_full=True)),
+                                                 (264, 64, 400, dict(a1_full=True)),
+                                                 (20, 256, 400, dict(rowwise=True)),
+                                                 (8, 512, 200, dict(rowwise=True))])
+def test_many_rows(srt, orc, mz, n_phi, n_ell, form):
+    """Enough rows to fill the GPU, so that the loop keeps two gathers in
+    flight."""
+    sz = dict(ms=8, mz=mz, dxy=0.4, dz=0.05, radius=6.0, n_phi=n_phi, n_zs=2, n_ell=n_ell)
+    _sample_check(srt, orc, sz, form, 1, 150, 30)

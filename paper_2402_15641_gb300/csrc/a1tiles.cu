@@ -46,7 +46,13 @@ __device__ unsigned long long g_viol;  // gathered rows outside their operand
 #endif
 
 // Records per group of the main loop; two groups alternate, as in tiles.cu.
-constexpr int kH = 3;
+// The loop is bound by the L1 data pipe and the gathers' latency; blocks of
+// four warps at 128 registers with the FMAs of a record under the test that
+// the slot's weight is not zero (see tiles.cu) take A1^T from 1.391 to 1.265
+// ms at 256^3, and groups of five where 128 columns leave the registers free
+// from 434 to 297 us at 128^3 (groups of three 346, four 328, six 307).
+template <int CH>
+constexpr int kH = CH == 2 ? 3 : 5;
 
 template <typename W>
 __device__ __forceinline__ void rec_w(const W* p, float w[4]);
@@ -100,12 +106,14 @@ struct A1Args {
 };
 
 
+constexpr int kNW = 4;  // warps of a block
+
 // Warp -> (group, index) as in spmm.cu's block_row: G groups of R, a block
-// owning TG groups x 8/TG consecutive indices, chunk-major, or S x S
+// owning TG groups x kNW/TG consecutive indices, chunk-major, or S x S
 // super-tiles (S > 0).
 __device__ __forceinline__ bool warp_tile(const A1Args& A, int* g, int* i) {
   const int w = threadIdx.x >> 5;
-  const int TI = 8 / A.TG;
+  const int TI = kNW / A.TG;
   if (A.S > 0) {
     const int per_row = A.S / A.TG, bpt = per_row * (A.S / TI);
     const int st = blockIdx.x / bpt, r = blockIdx.x - st * bpt;
@@ -161,7 +169,7 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
     SRT_CHECK_GATHER(0, row, A.xrows, g_viol);
     return row;
   };
-  constexpr int H = kH;
+  constexpr int H = kH<CH>;
   int oA[H], oB[H];
   float wA[H][4], wB[H][4];
   float4 vA[H][CH], vB[H][CH];
@@ -184,10 +192,9 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
     for (int u = 0; u < H; ++u)
 #pragma unroll
       for (int c = 0; c < CH; ++c)
-        if (in[c]) {
 #pragma unroll
-          for (int sg = 0; sg < 4; ++sg) fma4(acc[sym_slot(PS, PM, sg)][c], w[u][sg], v[u][c]);
-        }
+        for (int sg = 0; sg < 4; ++sg)
+          if (w[u][sg] != 0.f) fma4(acc[sym_slot(PS, PM, sg)][c], w[u][sg], v[u][c]);
   };
   int e = e0;
   const int groups = (e1 - e0) / H;
@@ -228,10 +235,9 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
 // f[b][p][k] = sum_(J,l) A1[(J, l), p] F1[b][(J, l)][k] for the 2 x 2 pixel
 // tile (ta, tb) with ta in [g0, g1); y points at pixel row 2 g0.
 template <typename W, int CH>
-__global__ void __launch_bounds__(256) k_a1t_tile(A1Args A, const W* __restrict__ wt,
-                                                  const float* __restrict__ x, int ldx,
-                                                  int64_t bsx, float* __restrict__ y, int ldy,
-                                                  int64_t bsy, int ncols) {
+__global__ void __launch_bounds__(kNW * 32, 4)
+    k_a1t_tile(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx, int64_t bsx,
+               float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
   const int lane = threadIdx.x & 31;
   int ga, tb;
   if (!warp_tile(A, &ga, &tb)) return;
@@ -376,7 +382,7 @@ namespace {
 template <typename W>
 int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t bsx, float* y,
                int64_t ldy, int64_t bsy, int ncols, int batch, cudaStream_t st) {
-  const int TI = 8 / A.TG;
+  const int TI = kNW / A.TG;
   int64_t gx;
   if (A.S > 0) {
     gx = (int64_t)((A.G + A.S - 1) / A.S) * ((A.R + A.S - 1) / A.S) * (A.S / A.TG) * (A.S / TI);
@@ -387,9 +393,9 @@ int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t
   const int CH = ncols > 128 ? 2 : 1;
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
   if (CH == 2)
-    k_a1t_tile<W, 2><<<grid, 256, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    k_a1t_tile<W, 2><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
   else
-    k_a1t_tile<W, 1><<<grid, 256, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    k_a1t_tile<W, 1><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }
@@ -417,15 +423,16 @@ int srt_a1tiles_apply(const srt_plan_s* plan, int g0, int g1, const float* x, in
   A.n_ell = g.n_ell;
   A.ntx = t.ntx;
   A.xrows = srt_checked_rows((int64_t)g.n_phi * g.n_ell);
-  // tiles (ta, tb), ta in [g0, g1): blocks of 4 x 2 tiles (8 x 4 pixels)
+  // tiles (ta, tb), ta in [g0, g1): blocks of 2 x 2 tiles (4 x 4 pixels)
   // walked in 16 x 16 tile (32 x 32 pixel) super-tiles where they fit, so
-  // the rows gathered at any time belong to a compact patch (1.457 ms at
-  // 256^3, against 1.483 with 32 x 32 tiles and 1.469 with none)
+  // the rows gathered at any time belong to a compact patch (with
+  // blocks of 4 x 2 tiles 1.457 ms at 256^3, against 1.483 with 32 x 32
+  // tiles and 1.469 with none; blocks of 4 x 1 tiles 1.276, of 2 x 2 1.272)
   A.g0 = g0;
   A.g1 = g1;
   A.G = g1 - g0;
   A.R = t.ntx;
-  A.TG = 4;
+  A.TG = 2;
   A.S = (A.G % 16 == 0 && A.R % 16 == 0) ? 16 : 0;
   if (g.weight_dtype == SRT_BF16) {
     const uint2* w = reinterpret_cast<const uint2*>(t.aw16);

@@ -242,13 +242,13 @@ int run_forward(srt_plan_s* p, const float* f, float* out, int B, float* w0, flo
     const int64_t ra = (int64_t)h0 * g.n_ell, rn = (int64_t)(h1 - h0) * g.n_ell;
     NvRange r("A2 product + reshape P2");
     if (fused_reshapes(p, nb)) {  // A2 tiles writing p[b][j][h][m] directly
-      SRT_TRY(srt_tiles_apply(p, false, h0, h1, 4, w1, nb, out, 0, (int)nb, st, r2));
+      SRT_TRY(srt_tiles_apply(p, false, h0, h1, w1, nb, out, 0, (int)nb, st, r2));
       if (!hs) mark(p, 0, 3, st);
       if (hs) SRT_TRY(sink_copy(hs, c, st, hs->host + ra, out + ra, rn, r2, (int64_t)B * g.n_phi));
       continue;
     }
     if (p->tiles && nb % 4 == 0)  // A2 from 2 x 2 tiles of the master tensor's taps
-      SRT_TRY(srt_tiles_apply(p, false, h0, h1, 4, w1, nb, w0 + ra * nb, nb, (int)nb, st));
+      SRT_TRY(srt_tiles_apply(p, false, h0, h1, w1, nb, w0 + ra * nb, nb, (int)nb, st));
     else if (p->toeplitz)  // A2 from the taps of the master tensor, a warp per row
       SRT_TRY(srt_taps_apply(p, false, ra, rn, h1 - h0, g.n_ell, 4, w1, nb, w0 + ra * nb, nb,
                              (int)nb, st));
@@ -287,9 +287,9 @@ int run_adjoint(srt_plan_s* p, const float* in, float* f, int B, float* w0, floa
   {
     NvRange r(fused ? "A2^T product + reshape P1^-1" : "A2^T product");
     if (fused)  // A2^T tiles writing F1[b][j][l][k] directly
-      SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, 4, w0, nb, w1, 0, (int)nb, st, c1));
+      SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, w0, nb, w1, 0, (int)nb, st, c1));
     else if (p->tiles && nb % 4 == 0)  // A2^T from 2 x 2 tiles of the master tensor's taps
-      SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, 4, w0, nb, w1, nb, (int)nb, st));
+      SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, w0, nb, w1, nb, (int)nb, st));
     else if (p->toeplitz)  // A2^T from the taps of the master tensor, a warp per row
       SRT_TRY(srt_taps_apply(p, true, 0, c1, 0, 0, 1, w0, nb, w1, nb, (int)nb, st));
     else

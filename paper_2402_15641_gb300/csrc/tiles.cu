@@ -90,20 +90,21 @@ __device__ __forceinline__ void tile_w<uint2>(const uint2* p, float w[4]) {
 // chunks together, so the rows gathered at any time stay in L2), from the
 // end of the radius range whose chunks hold more records: the last blocks
 // to start are then the light ones, and the SMs finish together.
-__device__ __forceinline__ void block_chunk(const TileArgs& A, int TG, int* ch, int* t) {
-  const int TI = 8 / TG;
+__device__ __forceinline__ void block_chunk(const TileArgs& A, int TG, int TI, int* ch, int* t) {
   const int tiles = (A.G + TG - 1) / TG;
   const int c = blockIdx.x / tiles;
   *t = blockIdx.x - c * tiles;
   *ch = A.desc ? (A.R + TI - 1) / TI - 1 - c : c;
 }
 
-// Tile of this warp: a block owns TG coordinate pairs x 8/TG radius pairs.
+// Tile of this warp: a block of NW warps owns TG coordinate pairs x NW/TG
+// radius pairs.
+template <int NW>
 __device__ __forceinline__ bool tile_of(const TileArgs& A, int* g, int* r) {
   const int w = threadIdx.x >> 5;
-  const int TI = 8 / A.TG;
+  const int TI = NW / A.TG;
   int ch, t;
-  block_chunk(A, A.TG, &ch, &t);
+  block_chunk(A, A.TG, TI, &ch, &t);
   *g = t * A.TG + w / TI;
   *r = ch * TI + w % TI;
   return *g < A.G && *r < A.R;
@@ -120,23 +121,36 @@ __device__ __forceinline__ void fma4(float2 (&a)[2], float w, const float4& xv) 
 // Records per group of the main loop.  The product waits on its gathers (L2
 // latency), so a warp alternates two groups: it requests the next group's
 // gathered rows before the FMAs of the current one, and its gathers stay in
-// flight while it computes.  At 128 registers and 16 warps per SM, groups
-// of three were fastest at 256^3 (A2 2.09 ms, A2^T 1.94 ms; a single group
-// of six whose FMAs wait for all its gathers: 2.24 / 2.06 ms; two groups
-// of two or of four: 3.20 / 3.29 and 3.60 / 4.20 ms; one record at a time,
-// 60 registers and 32 warps: 2.77 / 2.59 ms).
-constexpr int kTileH = 3;
+// flight while it computes.
+//
+// What bounds it, at 256 columns: the L1 data pipe, 94% busy (ncu).  A record
+// takes 8 cycles for its gathered row, 4 for its 16 bytes of weights (a
+// load that broadcasts from one address still writes every lane's registers)
+// and 1 for its offset, 44.1 M records a launch at 256^3: 1.82 ms.  The rest
+// is how the compiler orders the loop: the FMAs of a record run slot by slot
+// under the test that the slot's weight is not zero, which keeps each
+// group's loads ahead of the FMAs and its registers in reach (ms at 256^3,
+// A2 / A2^T: chunk by chunk without the test 2.06 / 1.94, slot by slot
+// without it 2.12 / 2.04, with it 1.93 / 1.85), at 128 registers in blocks of
+// four warps (of eight: 1.95 / 1.87).  Groups of two at 16 and 20 warps per
+// SM: 2.03 / 1.93 and 2.57 / 3.54, of four at 12: 2.00 / 1.89, one record at a
+// time at 24 warps: 2.24 / 2.15.  A true branch on the four tests (a jump
+// table): 2.70 / 2.57; weights through shared memory: 2.06 / 1.98.  With 128
+// columns or fewer half the registers hold rows, and groups of five fit (A2 /
+// A2^T at 64^3, 128 columns, us: three 49.2 / 46.1, five 45.2 / 44.2).
+template <int CH>
+constexpr int kTileH = CH == 2 ? 3 : 5;
 
 // Lanes own 4 consecutive dense columns of each of CH 128-column chunks.
 // TR: the block's outputs go through shared memory to the reshaped layout
 // (blocks of TG = 4 coordinate pairs x 2 radius pairs only).
 template <typename W, bool ADJ, int CH, bool TR>
-__global__ void __launch_bounds__(256) k_tile22(TileArgs A, const W* __restrict__ wt,
-                                                const float* __restrict__ x, int ldx,
-                                                float* __restrict__ y, int64_t ldy, int ncols) {
+__global__ void __launch_bounds__(TR ? 256 : 128, TR ? 2 : 4)
+    k_tile22(TileArgs A, const W* __restrict__ wt, const float* __restrict__ x, int ldx,
+             float* __restrict__ y, int64_t ldy, int ncols) {
   const int lane = threadIdx.x & 31;
   int g, r;
-  const bool mine = tile_of(A, &g, &r);
+  const bool mine = tile_of<TR ? 8 : 4>(A, &g, &r);
   if (!TR && !mine) return;  // (TR: every warp reaches the block barrier)
   const int c = A.c0 + 2 * g;
   const int n0 = blockIdx.y * (128 * CH) + lane * 4;
@@ -153,7 +167,7 @@ __global__ void __launch_bounds__(256) k_tile22(TileArgs A, const W* __restrict_
     const int e0 = pp[0], e1 = pp[A.E];
     const int64_t xb = ADJ ? (int64_t)c * A.n_ell : (int64_t)c;
     const float* x0 = x + xb * ldx + n0;
-    constexpr int H = kTileH;
+    constexpr int H = kTileH<CH>;
     int oA[H], oB[H];
     float wA[H][4], wB[H][4];
     float4 vA[H][CH], vB[H][CH];
@@ -179,10 +193,10 @@ __global__ void __launch_bounds__(256) k_tile22(TileArgs A, const W* __restrict_
 #pragma unroll
       for (int u = 0; u < H; ++u)
 #pragma unroll
-        for (int q = 0; q < CH; ++q)
-          if (in[q]) {
+        for (int s = 0; s < 4; ++s)
+          if (w[u][s] != 0.f) {
 #pragma unroll
-            for (int s = 0; s < 4; ++s) fma4(acc[s][q], w[u][s], v[u][q]);
+            for (int q = 0; q < CH; ++q) fma4(acc[s][q], w[u][s], v[u][q]);
           }
     };
     int e = e0;
@@ -246,7 +260,7 @@ __global__ void __launch_bounds__(256) k_tile22(TileArgs A, const W* __restrict_
   __shared__ __align__(16) float S[8 * 4 * 64];
   const int w = threadIdx.x >> 5;
   int ch, t;
-  block_chunk(A, 4, &ch, &t);
+  block_chunk(A, 4, 2, &ch, &t);
   const int cb = A.c0 + 8 * t, rb = 4 * ch;  // the block's first coordinate and radius
 #pragma unroll
   for (int pass = 0; pass < 2 * CH; ++pass) {
@@ -298,7 +312,7 @@ __global__ void __launch_bounds__(256) k_tile22(TileArgs A, const W* __restrict_
 template <typename W, bool ADJ>
 int launch(const TileArgs& A, const W* w, const float* x, int ldx, float* y, int64_t ldy,
            int ncols, cudaStream_t st) {
-  const int TI = 8 / A.TG;
+  const int TI = (A.ldn > 0 ? 8 : 4) / A.TG;
   const int64_t gx = (int64_t)((A.R + TI - 1) / TI) * ((A.G + A.TG - 1) / A.TG);
   if (gx > 0x7fffffff) return SRT_ERR_ARG;
   const int CH = ncols > 128 ? 2 : 1;
@@ -309,9 +323,9 @@ int launch(const TileArgs& A, const W* w, const float* x, int ldx, float* y, int
     else
       k_tile22<W, ADJ, 1, true><<<grid, 256, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
   } else if (CH == 2) {
-    k_tile22<W, ADJ, 2, false><<<grid, 256, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+    k_tile22<W, ADJ, 2, false><<<grid, 128, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
   } else {
-    k_tile22<W, ADJ, 1, false><<<grid, 256, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+    k_tile22<W, ADJ, 1, false><<<grid, 128, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
   }
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
@@ -431,7 +445,7 @@ int srt_build_tiles(srt_plan_s* plan, const std::vector<int32_t>& rp,
   return SRT_OK;
 }
 
-int srt_tiles_apply(const srt_plan_s* plan, bool adjoint, int c0, int c1, int TG, const float* x,
+int srt_tiles_apply(const srt_plan_s* plan, bool adjoint, int c0, int c1, const float* x,
                     int64_t ldx, float* y, int64_t ldy, int ncols, cudaStream_t st, int64_t ldn) {
   const srt_geometry& g = plan->g;
   const SrtTiles& t = adjoint ? plan->tla : plan->tlf;
@@ -439,8 +453,9 @@ int srt_tiles_apply(const srt_plan_s* plan, bool adjoint, int c0, int c1, int TG
   if (!t.ptr || c1 <= c0 || ncols <= 0 || ncols % 4 || ldx % 4 || (ldn <= 0 && ldy % 4) ||
       (uintptr_t)x % 16 || (uintptr_t)y % 16 || ldx > 0x7fffffff || ldn < 0)
     return SRT_ERR_ARG;
-  if (TG != 1 && TG != 2 && TG != 4 && TG != 8) TG = 4;
-  if (ldn > 0) TG = 4;  // the fused reshape stages blocks of 8 x 4 output rows
+  // blocks of 2 x 2 tiles (4 coordinates x 4 radii); the fused reshape
+  // stages blocks of 4 x 2 (8 x 4 output rows)
+  const int TG = ldn > 0 ? 4 : 2;
   TileArgs A{t.ptr, t.off, t.nkeys, t.key0, adjoint ? g.n_zs : g.mz, c0, c1, g.n_ell, g.mz,
              (c1 - c0 + 1) / 2, t.pairs, TG, t.desc ? 1 : 0,
              srt_checked_rows(adjoint ? (int64_t)g.n_zs * g.n_ell : (int64_t)g.n_ell * g.mz),

@@ -30,7 +30,8 @@
 // and D map aligned 2 x 2 tiles to aligned 2 x 2 tiles when ms is even),
 // whose records (j, l), sorted by (list, j, l), gather row (C_g(j), l) of F1
 // into the output pixel P_g(q_sigma) of T: a fixed permutation of the
-// tile's four slots per g.  With every column stored (one pass) each pixel
+// tile's four slots per g (with few slabs the warp's groups of lanes share
+// the elements, k_a1t_split).  With every column stored (one pass) each pixel
 // sums its entries in the CSR order of A1^T, ascending (j, l).  Every output
 // row is one warp's FP32 sum: no atomics, deterministic.
 #include <algorithm>
@@ -277,6 +278,152 @@ __global__ void __launch_bounds__(kNW * 32, 4)
   }
 }
 
+// One FP32 weight of a record (slot q).
+__device__ __forceinline__ float rec_w1(const float4* p, int q) {
+  return __ldg(reinterpret_cast<const float*>(p) + q);
+}
+__device__ __forceinline__ float rec_w1(const uint2* p, int q) {
+  return srt_bf16_to_f32(__ldg(reinterpret_cast<const uint16_t*>(p) + q));
+}
+
+// A1^T with at most 64 slabs from a symmetric form: GL lanes cover the width
+// and the warp's 32 / GL groups of lanes take the group elements of the same
+// tile between them (the 8-fold form's 8 passes, the quarter turns' 4), so
+// no lane idles and a tile's chain of gathers is 32 / GL times shorter.  Each
+// group permutes a record's weights as it loads them, four 4-byte loads
+// that cost the L1 data pipe no more than one 16-byte load, and the groups'
+// sums are added at the end.  us, a whole warp to a pass before: 16^3 22.5 ->
+// 10.2 (GL = 4), 48^3 38.9 -> 26.6, 64^3 63.5 -> 45.1 (GL = 16; GL = 8 with two
+// chunks 45.1, 28.7 at 48^3).  With 96 or 128 slabs two chunks a lane leave
+// too few registers for groups of five: 201 against 166 and 350 against 297
+// us, so wider volumes keep a warp to a pass.
+template <typename W, int CH, int GL>
+__global__ void __launch_bounds__(kNW * 32, 4)
+    k_a1t_split(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx,
+                int64_t bsx, float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
+  constexpr int NS = 32 / GL, H = kH<CH>;
+  const int lane = threadIdx.x & 31, sub = lane / GL, sl = lane % GL;
+  int ga, tb;
+  if (!warp_tile(A, &ga, &tb)) return;
+  const int ta = A.g0 + ga;
+  const int n0 = sl * 4;
+  const float* x0 = x + blockIdx.z * bsx + n0;
+  bool in[CH];
+#pragma unroll
+  for (int c = 0; c < CH; ++c) in[c] = n0 + c * (4 * GL) < ncols;
+  float2 acc[4][CH][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < CH; ++c) acc[i][c][0] = acc[i][c][1] = make_float2(0.f, 0.f);
+  const int np = A.mode == 2 ? 8 : 4;
+#pragma unroll 1
+  for (int pi = 0; pi < np; pi += NS) {
+    // this group's element g = rot^ps D^pm, its stored tile and its column map
+    const int pg = pi + sub, ps = pg & 3, pm = pg >> 2;
+    const int n = A.ntx - 1;
+    int qa = ps == 0 ? ta : ps == 1 ? tb : ps == 2 ? n - ta : n - tb;
+    int qb = ps == 0 ? tb : ps == 1 ? n - ta : ps == 2 ? n - tb : ta;
+    if (pm) {
+      const int t = qa;
+      qa = qb;
+      qb = t;
+    }
+    const int64_t t2 = 2 * ((int64_t)qa * A.ntx + qb);
+    const int e0 = A.ptr[t2], e1 = pg < np ? A.ptr[t2 + (pm ? 1 : 2)] : e0;
+    const int cnt = e1 - e0, most = (int)__reduce_max_sync(0xffffffffu, (unsigned)cnt);
+    const int base = (ps + pm) * A.q, sign = pm ? -1 : 1;
+    int from[4];  // stored slot that lands in slot d
+#pragma unroll
+    for (int sg = 0; sg < 4; ++sg) from[sg] = 0;
+#pragma unroll
+    for (int sg = 0; sg < 4; ++sg) {
+      const int d = sym_slot(ps, pm, sg);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k == d) from[k] = sg;
+    }
+    {  // the pass's records from L2 at once, as in a1t_pass
+      const char* kb = reinterpret_cast<const char*>(A.key + e0);
+      for (int b = sl * 128; b < cnt * 4; b += GL * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(kb + b));
+      const char* wb = reinterpret_cast<const char*>(wt + e0);
+      for (int b = sl * 128; b < cnt * (int)sizeof(W); b += GL * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(wb + b));
+    }
+    float wA[H][4], wB[H][4];
+    float4 vA[H][CH], vB[H][CH];
+    // records eb .. eb + H - 1 of each group's own list; past its end the
+    // last record again, with zero weights
+    auto load = [&](int eb, float (&w)[H][4], float4 (&v)[H][CH]) {
+      int o[H];
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const int k = __ldg(A.key + max(0, e0 + min(eb + u, cnt - 1)));
+        int J = base + sign * (k >> 16);
+        if (J >= A.n_phi) J -= A.n_phi;
+        o[u] = J * A.n_ell + (k & 0xffff);
+        SRT_CHECK_GATHER(0, o[u], A.xrows, g_viol);
+      }
+#pragma unroll
+      for (int u = 0; u < H; ++u) {
+        const float* xr = x0 + (int64_t)o[u] * ldx;
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (in[c]) v[u][c] = srt_ldg_keep(xr + c * (4 * GL));
+      }
+#pragma unroll
+      for (int u = 0; u < H; ++u)
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+          w[u][d] = eb + u < cnt ? rec_w1(wt + e0 + eb + u, from[d]) : 0.f;
+    };
+    auto comp = [&](float (&w)[H][4], float4 (&v)[H][CH]) {
+#pragma unroll
+      for (int u = 0; u < H; ++u)
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+          for (int d = 0; d < 4; ++d)
+            if (w[u][d] != 0.f) fma4(acc[d][c], w[u][d], v[u][c]);
+    };
+    if (most > 0) {
+      load(0, wA, vA);
+#pragma unroll 1
+      for (int r = 0; r < most; r += 2 * H) {
+        load(r + H, wB, vB);
+        comp(wA, vA);
+        load(r + 2 * H, wA, vA);
+        comp(wB, vB);
+      }
+    }
+  }
+  // the groups' sums, added in a fixed tree
+#pragma unroll
+  for (int o = GL; o < 32; o <<= 1)
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+      for (int c = 0; c < CH; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          acc[d][c][h].x += __shfl_xor_sync(0xffffffffu, acc[d][c][h].x, o);
+          acc[d][c][h].y += __shfl_xor_sync(0xffffffffu, acc[d][c][h].y, o);
+        }
+  float* y0 = y + blockIdx.z * bsy;
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    if (d % NS != sub) continue;  // one group stores each slot
+    const int ix = 2 * ga + (d >> 1), iy = 2 * tb + (d & 1);  // ix relative to row 2 g0
+    float* yr = y0 + ((int64_t)ix * A.ms + iy) * ldy;
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      if (in[c])
+        *reinterpret_cast<float4*>(yr + n0 + c * (4 * GL)) =
+            make_float4(acc[d][c][0].x, acc[d][c][0].y, acc[d][c][1].x, acc[d][c][1].y);
+  }
+}
+
 // ------------------------------------------------------------ records
 struct TEnt {
   int64_t key;  // list << 40 | j << 16 | l
@@ -390,6 +537,17 @@ int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t
     gx = (int64_t)((A.R + TI - 1) / TI) * ((A.G + A.TG - 1) / A.TG);
   }
   if (gx > 0x7fffffff || batch > 65535) return SRT_ERR_ARG;
+  if (A.mode && ncols <= 64) {
+    dim3 grid((unsigned)gx, 1, batch);
+    if (ncols <= 16 && A.mode == 2)  // 8 groups: one to each of the 8 passes
+      k_a1t_split<W, 1, 4><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    else if (ncols <= 32)
+      k_a1t_split<W, 1, 8><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    else
+      k_a1t_split<W, 1, 16><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    SRT_CUDA_TRY(cudaGetLastError());
+    return SRT_OK;
+  }
   const int CH = ncols > 128 ? 2 : 1;
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
   if (CH == 2)

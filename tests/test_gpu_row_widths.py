@@ -56,3 +56,21 @@ def test_many_rows(srt, orc, mz, n_phi, n_ell, form):
     flight."""
     sz = dict(ms=8, mz=mz, dxy=0.4, dz=0.05, radius=6.0, n_phi=n_phi, n_zs=2, n_ell=n_ell)
     _sample_check(srt, orc, sz, form, 1, 150, 30)
+
+
+@pytest.mark.parametrize("mz", [4, 16, 20, 32, 36, 64, 68])
+@pytest.mark.parametrize("form", [dict(), dict(a1_rotation=True), dict(weight_dtype="bf16")])
+def test_adjoint_group_passes(srt, orc, mz, form):
+    """A1^T with the symmetry passes shared by a warp's groups of lanes (at
+    most 64 slabs: 4, 8 and 16 lanes to a group; quarter turns keep 8) and
+    with a warp to a pass (68), batch 3, an odd number of tiles."""
+    sz = dict(ms=10, mz=mz, dxy=0.4, dz=0.4, radius=6.0, n_phi=16, n_zs=3, n_ell=21)
+    bf16 = form.get("weight_dtype") == "bf16"
+    g, o = geom_pair(orc, **form, **sz)
+    plan = srt.Plan(g)
+    assert plan.info["a1_rot"] == (1 if form.get("a1_rotation") else 2)
+    y = np.random.default_rng(63).standard_normal((3, *g.p_shape)).astype(np.float32)
+    a = to_np(plan.adjoint(to_dev(y)))
+    for b in range(3):
+        want = orc.adjoint(o, y[b].astype(np.float64))
+        assert rel_l2(a[b], want) <= (5e-3 if bf16 else 1e-5)

@@ -239,6 +239,7 @@ template <typename W, int CH>
 __global__ void __launch_bounds__(kNW * 32, 4)
     k_a1t_tile(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx, int64_t bsx,
                float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
+  srt_in_order();
   const int lane = threadIdx.x & 31;
   int ga, tb;
   if (!warp_tile(A, &ga, &tb)) return;
@@ -301,6 +302,7 @@ template <typename W, int CH, int GL>
 __global__ void __launch_bounds__(kNW * 32, 4)
     k_a1t_split(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx,
                 int64_t bsx, float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
+  srt_in_order();
   constexpr int NS = 32 / GL, H = kH<CH>;
   const int lane = threadIdx.x & 31, sub = lane / GL, sl = lane % GL;
   int ga, tb;
@@ -540,20 +542,25 @@ int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t
   if (A.mode && ncols <= 64) {
     dim3 grid((unsigned)gx, 1, batch);
     if (ncols <= 16 && A.mode == 2)  // 8 groups: one to each of the 8 passes
-      k_a1t_split<W, 1, 4><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 4>, grid, kNW * 32, st, A, w, x, (int)ldx,
+                              bsx, y, (int)ldy, bsy, ncols));
     else if (ncols <= 32)
-      k_a1t_split<W, 1, 8><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 8>, grid, kNW * 32, st, A, w, x, (int)ldx,
+                              bsx, y, (int)ldy, bsy, ncols));
     else
-      k_a1t_split<W, 1, 16><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 16>, grid, kNW * 32, st, A, w, x,
+                              (int)ldx, bsx, y, (int)ldy, bsy, ncols));
     SRT_CUDA_TRY(cudaGetLastError());
     return SRT_OK;
   }
   const int CH = ncols > 128 ? 2 : 1;
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
   if (CH == 2)
-    k_a1t_tile<W, 2><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_tile<W, 2>, grid, kNW * 32, st, A, w, x, (int)ldx, bsx,
+                            y, (int)ldy, bsy, ncols));
   else
-    k_a1t_tile<W, 1><<<grid, kNW * 32, 0, st>>>(A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, ncols);
+    SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_tile<W, 1>, grid, kNW * 32, st, A, w, x, (int)ldx, bsx,
+                            y, (int)ldy, bsy, ncols));
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }

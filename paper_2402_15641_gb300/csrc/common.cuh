@@ -113,6 +113,8 @@ struct SrtA1Tiles {
   uint16_t* aw16 = nullptr; // 4 * na (SRT_BF16)
 };
 
+constexpr int kSMs = 152;
+
 struct SrtHostPool;  // copy streams and events of host-buffer calls (api.cu)
 
 struct srt_plan_s {
@@ -215,7 +217,49 @@ int srt_transpose(const float* in, int64_t ild, int64_t ibs, float* out, int64_t
 
 int srt_dot(const float* a, const float* b, int64_t n, double* out, double* partials,
             cudaStream_t stream);
-constexpr int SRT_DOT_BLOCKS = 608;  // 152 SMs x 4
+constexpr int SRT_DOT_BLOCKS = 4 * kSMs;
+
+// ------------------------------------------------------ launches in sequence
+// The kernels of a call depend each on the one before.  A small one is
+// launched with programmatic stream serialization: its blocks may become
+// resident while the kernel before still runs, and srt_in_order(), the first
+// statement of every kernel here, waits until that kernel has completed and
+// its writes are visible.  Only then does it let the next kernel's blocks
+// come up, so at most one kernel waits ahead, and it was launched (its L1
+// lines dropped) after every earlier reader of its operand had finished.
+// Without the attribute both instructions do nothing.  Work that follows a
+// call in its stream waits for the last kernel as usual.
+//
+// What is gained is the launch latency between two kernels, about a
+// microsecond; what it costs is room on the SMs at the end of the kernel
+// before.  So `early` says up to how many blocks a kernel is launched so
+// (forward, pair or adjoint, us, without and with): 32^3 30.8 and 26.8, 64^3
+// 95.1 and 92.2, a 75 x 75 x 53 pair 140 and 130; beyond the limits given at
+// each launch calls got slower (96^3 adjoint 355 and 360 with its 576 A1^T
+// blocks early, 256^3 forward 3547 and 3729 with every kernel early), and the
+// 64 x 64 tile reshapes, whose 17 KB of shared memory a block takes from the
+// L1 of the kernel before, are never early.
+__device__ __forceinline__ void srt_in_order() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t srt_launch(int early, void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st,
+                              A... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = (int64_t)grid.x * grid.y * grid.z <= early ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 
 // --------------------------------------------------- FP64 device helpers
 // Angle in [0, pi] whose cosine is u/r, clamped at the ends.  The sine side

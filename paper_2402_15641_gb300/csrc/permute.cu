@@ -12,6 +12,7 @@ constexpr int TILE = 32;
 __global__ void __launch_bounds__(256) k_transpose(const float* __restrict__ in, int64_t ild,
                                                    int64_t ibs, float* __restrict__ out,
                                                    int64_t old, int64_t obs, int rows, int cols) {
+  srt_in_order();
   __shared__ float tile[TILE][TILE + 1];
   in += blockIdx.z * ibs;
   out += blockIdx.z * obs;
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(256) k_transpose_v4(const float* __restrict__ 
                                                       int64_t ibs, float* __restrict__ out,
                                                       int64_t old, int64_t obs, int rows,
                                                       int cols) {
+  srt_in_order();
   __shared__ float tile[VT][VT + 1];
   in += blockIdx.z * ibs;
   out += blockIdx.z * obs;
@@ -106,14 +108,16 @@ int srt_transpose(const float* in, int64_t ild, int64_t ibs, float* out, int64_t
   if (v4) {
     dim3 grid((cols + VT - 1) / VT, (rows + VT - 1) / VT, batch);
     if (grid.y > 65535 || grid.z > 65535) return SRT_ERR_ARG;
-    k_transpose_v4<<<grid, 256, 0, st>>>(in, ild, ibs, out, old, obs, rows, cols);
+    SRT_CUDA_TRY(srt_launch(0, k_transpose_v4, grid, 256, st, in, ild, ibs, out, old, obs, rows,
+                            cols));
     SRT_CUDA_TRY(cudaGetLastError());
     return SRT_OK;
   }
   dim3 block(TILE, 8);
   dim3 grid((cols + TILE - 1) / TILE, (rows + TILE - 1) / TILE, batch);
   if (grid.y > 65535 || grid.z > 65535) return SRT_ERR_ARG;
-  k_transpose<<<grid, block, 0, st>>>(in, ild, ibs, out, old, obs, rows, cols);
+  SRT_CUDA_TRY(srt_launch(16 * kSMs, k_transpose, grid, block, st, in, ild, ibs, out, old, obs,
+                          rows, cols));
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }

@@ -22,7 +22,6 @@
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int kSMs = 152;
 #ifdef SRT_CHECKS
 __device__ unsigned long long g_viol;  // gathered rows outside their operand
 #endif
@@ -153,6 +152,7 @@ __global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* _
                                               int64_t bsy, int ncols, int G, int R, int TG, int S,
                                               int ms, int n_ell, int q, int mirror,
                                               uint64_t magic, int xrows, int64_t ldn) {
+  srt_in_order();
   constexpr int NR = 32 / GL, EB = GL == 32 ? 32 : 16;
   // 384 or 512 columns to a warp: the pairs stay in registers and go round
   // by shuffles, whose share of the row's time is small there, and the
@@ -334,9 +334,10 @@ int launch_as(const SrtCsr& A, const V* val, const Rows& W, const float* x, int6
   if (gx > 0x7fffffff || (ncols + wide - 1) / wide > 65535 || batch > 65535) return SRT_ERR_ARG;
   dim3 grid((unsigned)gx, (ncols + wide - 1) / wide, batch);
   const SrtRot& r = W.rot;
-  k_rows<V, VW, CH, GL, MODE, TR, U><<<grid, 256, 0, st>>>(
-      W.rows, W.r0, A.rowptr, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R, W.TG, S, r.ms,
-      r.n_ell, r.q, r.mirror, W.magic, W.xrows, W.ldn);
+  SRT_CUDA_TRY(srt_launch(12 * kSMs, k_rows<V, VW, CH, GL, MODE, TR, U>, grid, 256, st, W.rows,
+                          W.r0, A.rowptr, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R,
+                          W.TG, S, r.ms,
+      r.n_ell, r.q, r.mirror, W.magic, W.xrows, W.ldn));
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }

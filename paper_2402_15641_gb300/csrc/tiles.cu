@@ -148,6 +148,7 @@ template <typename W, bool ADJ, int CH, bool TR>
 __global__ void __launch_bounds__(TR ? 256 : 128, TR ? 2 : 4)
     k_tile22(TileArgs A, const W* __restrict__ wt, const float* __restrict__ x, int ldx,
              float* __restrict__ y, int64_t ldy, int ncols) {
+  srt_in_order();
   const int lane = threadIdx.x & 31;
   int g, r;
   const bool mine = tile_of<TR ? 8 : 4>(A, &g, &r);
@@ -319,13 +320,17 @@ int launch(const TileArgs& A, const W* w, const float* x, int ldx, float* y, int
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), 1);
   if (A.ldn > 0) {
     if (CH == 2)
-      k_tile22<W, ADJ, 2, true><<<grid, 256, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+      SRT_CUDA_TRY(srt_launch(8 * kSMs, k_tile22<W, ADJ, 2, true>, grid, 256, st, A, w, x, ldx, y,
+                              ldy, ncols));
     else
-      k_tile22<W, ADJ, 1, true><<<grid, 256, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+      SRT_CUDA_TRY(srt_launch(8 * kSMs, k_tile22<W, ADJ, 1, true>, grid, 256, st, A, w, x, ldx, y,
+                              ldy, ncols));
   } else if (CH == 2) {
-    k_tile22<W, ADJ, 2, false><<<grid, 128, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+    SRT_CUDA_TRY(srt_launch(8 * kSMs, k_tile22<W, ADJ, 2, false>, grid, 128, st, A, w, x, ldx, y,
+                            ldy, ncols));
   } else {
-    k_tile22<W, ADJ, 1, false><<<grid, 128, 0, st>>>(A, w, x, ldx, y, ldy, ncols);
+    SRT_CUDA_TRY(srt_launch(8 * kSMs, k_tile22<W, ADJ, 1, false>, grid, 128, st, A, w, x, ldx, y,
+                            ldy, ncols));
   }
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;

@@ -80,6 +80,7 @@ template <typename V, int CH, bool ADJ>
 __global__ void __launch_bounds__(256) k_taps(TapArgs A, const V* __restrict__ val,
                                               const float* __restrict__ x, int64_t ldx,
                                               float* __restrict__ y, int64_t ldy, int ncols) {
+  srt_in_order();
   const int lane = threadIdx.x & 31;
   const int lr = tap_row(A.G, A.R, A.TG);
   if (lr < 0 || lr >= A.rows) return;
@@ -148,6 +149,7 @@ __global__ void __launch_bounds__(256) k_taps_scalar(TapArgs A, const V* __restr
                                                      const float* __restrict__ x, int64_t ldx,
                                                      float* __restrict__ y, int64_t ldy,
                                                      int ncols) {
+  srt_in_order();
   const int lane = threadIdx.x & 31;
   const int lr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (lr >= A.rows) return;
@@ -198,7 +200,8 @@ int launch(const TapArgs& A, const V* val, const float* x, int64_t ldx, float* y
                    (uintptr_t)y % 16 == 0;
   if (!vec) {
     dim3 grid((unsigned)(((int64_t)A.rows + 7) / 8), (ncols + 127) / 128, 1);
-    k_taps_scalar<V, 4, ADJ><<<grid, 256, 0, st>>>(A, val, x, ldx, y, ldy, ncols);
+    SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps_scalar<V, 4, ADJ>, grid, 256, st, A, val, x, ldx, y,
+                            ldy, ncols));
     SRT_CUDA_TRY(cudaGetLastError());
     return SRT_OK;
   }
@@ -210,10 +213,14 @@ int launch(const TapArgs& A, const V* val, const float* x, int64_t ldx, float* y
   const int CH = chunks >= 4 ? 4 : chunks;
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), 1);
   switch (CH) {
-    case 4: k_taps<V, 4, ADJ><<<grid, 256, 0, st>>>(A, val, x, ldx, y, ldy, ncols); break;
-    case 3: k_taps<V, 3, ADJ><<<grid, 256, 0, st>>>(A, val, x, ldx, y, ldy, ncols); break;
-    case 2: k_taps<V, 2, ADJ><<<grid, 256, 0, st>>>(A, val, x, ldx, y, ldy, ncols); break;
-    default: k_taps<V, 1, ADJ><<<grid, 256, 0, st>>>(A, val, x, ldx, y, ldy, ncols); break;
+    case 4: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 4, ADJ>, grid, 256, st, A, val, x, ldx, y,
+                                    ldy, ncols)); break;
+    case 3: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 3, ADJ>, grid, 256, st, A, val, x, ldx, y,
+                                    ldy, ncols)); break;
+    case 2: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 2, ADJ>, grid, 256, st, A, val, x, ldx, y,
+                                    ldy, ncols)); break;
+    default: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 1, ADJ>, grid, 256, st, A, val, x, ldx, y,
+                                     ldy, ncols)); break;
   }
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;

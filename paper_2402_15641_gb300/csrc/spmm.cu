@@ -116,6 +116,11 @@ __device__ __forceinline__ void ld_cols(const float* p, float (&v)[VW]) {
   }
 }
 
+// Warps of a block (four where a warp holds four rows or more: 8 x 64^3 224 ->
+// 217 us, 96^3 185 -> 180).
+template <int GL>
+constexpr int kBlockWarps = GL > 8 ? 8 : 4;
+
 // A group of GL lanes owns an output row, 32 / GL rows to a warp; a lane
 // owns VW consecutive columns of each of CH chunks of VW GL columns.  The
 // row's entries are loaded EB at a time by the group's lanes, the gathered
@@ -130,11 +135,13 @@ __device__ __forceinline__ void ld_cols(const float* p, float (&v)[VW]) {
 // where each entry takes 8 cycles for its 1 KB and 2 for broadcasting row
 // and value by two shuffles.  The pair read back by one 8-byte shared load
 // takes 1 (a load that all lanes read from one shared address costs half of
-// what it writes to registers): A1 at 256^3 1.578 -> 1.526 ms.  Below 128
+// what it writes to registers): A1 at 256^3 1.578 -> 1.526 ms, and 1.480 with
+// each batch's entries requested before the batch before is gathered (8 x
+// 64^3 218 -> 212 us, 128^3 346 -> 340, 192^3 1088 -> 1072).  Below 128
 // columns a whole warp to a row leaves lanes idle and spends the same loop
 // on fewer columns; with GL lanes to a row (measured, one box, FP32 entries,
-// a warp to a row before): 8 x 64^3 446 -> 224 us, 128^3 416 -> 346, 192^3
-// 1180 -> 1089.  U gathers are requested before their FMAs: two cost no
+// a warp to a row before): 8 x 64^3 446 -> 212 us, 128^3 416 -> 340, 192^3
+// 1180 -> 1072.  U gathers are requested before their FMAs: two cost no
 // registers' worth of residency (32, 64 warps per SM) and gain 4% at 128^3;
 // four cost 6% at 256^3 but win where the launch cannot fill the GPU.
 // A row's entries are summed in the same order in every variant.
@@ -144,14 +151,11 @@ __device__ __forceinline__ void ld_cols(const float* p, float (&v)[VW]) {
 // shared memory, 128 slabs at a time, and are written as Y1'[(l, k)][b G +
 // j], row stride ldn, 16 bytes (4 sensor columns) per radius and slab.
 template <typename V, int VW, int CH, int GL, int MODE, bool TR, int U>
-__global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* __restrict__ rowptr,
-                                              const int32_t* __restrict__ col,
-                                              const V* __restrict__ val,
-                                              const float* __restrict__ x, int64_t ldx,
-                                              int64_t bsx, float* __restrict__ y, int64_t ldy,
-                                              int64_t bsy, int ncols, int G, int R, int TG, int S,
-                                              int ms, int n_ell, int q, int mirror,
-                                              uint64_t magic, int xrows, int64_t ldn) {
+__global__ void __launch_bounds__(kBlockWarps<GL> * 32)
+    k_rows(int rows, int r0, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+           const V* __restrict__ val, const float* __restrict__ x, int64_t ldx, int64_t bsx,
+           float* __restrict__ y, int64_t ldy, int64_t bsy, int ncols, int G, int R, int TG, int S,
+           int ms, int n_ell, int q, int mirror, uint64_t magic, int xrows, int64_t ldn) {
   srt_in_order();
   constexpr int NR = 32 / GL, EB = GL == 32 ? 32 : 16;
   // 384 or 512 columns to a warp: the pairs stay in registers and go round
@@ -159,9 +163,9 @@ __global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* _
   // shared loads' extra registers cost more (A2 as CSR at 3072 columns 244
   // us, 268 through shared memory; A2^T 249, 316)
   constexpr bool SH = GL == 32 && VW == 4 && CH > 2;
-  __shared__ int2 stage[SH ? 1 : 8][NR][EB + (NR > 1 ? 1 : 0)];
+  __shared__ int2 stage[SH ? 1 : kBlockWarps<GL>][NR][EB + (NR > 1 ? 1 : 0)];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane / GL, sl = lane % GL;
-  const int lr = block_row<8 * NR>(G, R, TG, S, w * NR + sub);
+  const int lr = block_row<kBlockWarps<GL> * NR>(G, R, TG, S, w * NR + sub);
   const bool mine = lr >= 0 && lr < rows;
   if (!TR && NR == 1 && !mine) return;  // (otherwise every lane reaches the barriers)
   const int row = r0 + (mine ? lr : 0);
@@ -191,8 +195,23 @@ __global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* _
     if (MODE == 2) sr = rot_pixel(row, 4 - s, ms, magic);
     const int off = MODE == 2 ? s * q * n_ell : 0;
     const int e0 = rowptr[sr], e1 = mine ? rowptr[sr + 1] : e0;
-    // batches run in step over the warp's rows (an exhausted row idles)
+    // batches run in step over the warp's rows (an exhausted row idles); the
+    // next batch's entries are requested before this one's gathers
     const int len = NR > 1 ? (int)__reduce_max_sync(FULL, (unsigned)(e1 - e0)) : e1 - e0;
+    constexpr int KE = EB / GL;
+    // (short rows of single columns have too few gathers to cover the request)
+    constexpr bool PF = !SH && !(VW == 1 && U == 4);
+    int nc[KE];
+    V nv[KE];
+    auto ask = [&](int eb) {
+#pragma unroll
+      for (int k = 0; k < KE; ++k)
+        if (eb + sl + k * GL < e1) {
+          nc[k] = col[eb + sl + k * GL];
+          nv[k] = val[eb + sl + k * GL];
+        }
+    };
+    if (PF) ask(e0);
 #pragma unroll 1
     for (int b = 0; b < len; b += EB) {
       const int eb = e0 + b;
@@ -225,16 +244,17 @@ __global__ void __launch_bounds__(256) k_rows(int rows, int r0, const int32_t* _
         }
         continue;
       }
+      if (!PF) ask(eb);
 #pragma unroll
-      for (int i = sl; i < EB; i += GL) {
-        if (eb + i < e1) {
-          int c = col[eb + i];
+      for (int k = 0; k < KE; ++k)
+        if (eb + sl + k * GL < e1) {
+          int c = nc[k];
           if (MODE == 1) c = rot_pixel(c, t, ms, magic, mir);
           if (MODE == 2) c += off;
           SRT_CHECK_GATHER(0, c, xrows, g_viol);
-          st[i] = make_int2(c, __float_as_int(wval<V>(val[eb + i])));
+          st[sl + k * GL] = make_int2(c, __float_as_int(wval<V>(nv[k])));
         }
-      }
+      if (PF) ask(eb + EB);
       __syncwarp();
       const int cnt = min(EB, e1 - eb);
       int i = 0;
@@ -324,7 +344,7 @@ template <typename V, int VW, int CH, int GL, int MODE, int U, bool TR = false>
 int launch_as(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t ldx,
               int64_t bsx, float* y, int64_t ldy, int64_t bsy, int ncols, int batch,
               cudaStream_t st) {
-  constexpr int RPB = 8 * (32 / GL);
+  constexpr int RPB = kBlockWarps<GL> * (32 / GL);
   const int TI = RPB / W.TG;
   const int S = W.S > 0 && W.S % TI == 0 ? W.S : 0;
   const int64_t gx = S > 0     ? (int64_t)(W.G / S) * (W.R / S) * (S / W.TG) * (S / TI)
@@ -334,7 +354,7 @@ int launch_as(const SrtCsr& A, const V* val, const Rows& W, const float* x, int6
   if (gx > 0x7fffffff || (ncols + wide - 1) / wide > 65535 || batch > 65535) return SRT_ERR_ARG;
   dim3 grid((unsigned)gx, (ncols + wide - 1) / wide, batch);
   const SrtRot& r = W.rot;
-  SRT_CUDA_TRY(srt_launch(12 * kSMs, k_rows<V, VW, CH, GL, MODE, TR, U>, grid, 256, st, W.rows,
+  SRT_CUDA_TRY(srt_launch(12 * kSMs, k_rows<V, VW, CH, GL, MODE, TR, U>, grid, kBlockWarps<GL> * 32, st, W.rows,
                           W.r0, A.rowptr, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R,
                           W.TG, S, r.ms,
       r.n_ell, r.q, r.mirror, W.magic, W.xrows, W.ldn));

@@ -335,8 +335,7 @@ int g_checks_cap = 0;
 
 long long checks_take_all() {
   long long n = 0;
-  for (long long v : {srt_checks_take_spmm(), srt_checks_take_taps(), srt_checks_take_tiles(),
-                      srt_checks_take_a1tiles()}) {
+  for (long long v : {srt_checks_take_spmm(), srt_checks_take_tiles(), srt_checks_take_a1tiles()}) {
     if (v < 0) return -1;
     n += v;
   }

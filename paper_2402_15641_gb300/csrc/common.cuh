@@ -36,7 +36,6 @@
 // Violations counted by each translation unit's kernels since the last
 // call, then reset (0 in release builds), and the row cap of srt_checks_cap.
 long long srt_checks_take_spmm();
-long long srt_checks_take_taps();
 long long srt_checks_take_tiles();
 long long srt_checks_take_a1tiles();
 int srt_checks_rowcap();
@@ -191,10 +190,12 @@ int srt_a1tiles_apply(const srt_plan_s* plan, int g0, int g1, const float* x, in
 // mirror: column s q + t from stored column q - t for t > q/2, pixels
 // mirrored across the diagonal first);
 // mode 2 = A1^T rows (pixels) from 4 stored rows of the stored transpose.
+// mode 3, 4 = A2 rows (h, m) and A2^T rows (l, k) from the Toeplitz taps
+// (toeplitz.cu), with ms = mz and q = n_zs.
 struct SrtRot {
   int mode = 0;           // 0: rows are stored as they are
   int ms = 0, n_ell = 0;  // pixel grid edge, radius bins
-  int q = 0;              // n_phi / 4
+  int q = 0;              // n_phi / 4 (modes 3, 4: n_zs)
   int mirror = 0;         // mode 1 only: the 8-fold form (stored columns 0 .. q/2)
 };
 

@@ -127,8 +127,10 @@ constexpr int kBlockWarps = GL > 8 ? 8 : 4;
 // row remapped there (MODE 1: A1 row (j, l) from stored row (j mod q, l),
 // pixels turned j / q times, mirrored first where the stored column is a
 // mirror image; MODE 2: A1^T row p from stored rows rot^-s(p), s = 0..3,
-// gathered rows shifted by s q n_ell), and put in shared memory as (row,
-// value) pairs that the group then reads back.
+// gathered rows shifted by s q n_ell; MODE 3 and 4: A2 rows (h, m) and A2^T
+// rows (l, k) from the Toeplitz taps, ms = mz slabs and q = n_zs rings, see
+// toeplitz.cu), and put in shared memory as (row, value) pairs that the group
+// then reads back.
 //
 // What bounds it.  A gathered operand feeds one FMA, so the L1 data pipe
 // (128 B a cycle per SM) is the limit at full width: 93% busy at 256^3,
@@ -177,8 +179,18 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32)
   for (int k = 0; k < CH; ++k)
 #pragma unroll
     for (int i = 0; i < VW; ++i) acc[k][i] = 0.f;
-  int t = 0, sr = row;
+  int t = 0, sr = row, ca = 0;
   bool mir = false;
+  if (MODE == 3) {  // taps of row (h, m): offsets nz-1-h .. of radius m, row l mz + h + q-(nz-1)
+    const int h = row / n_ell, m = row - h * n_ell;
+    sr = m * (ms + q - 1) + q - 1 - h;
+    ca = h - (q - 1);
+  }
+  if (MODE == 4) {  // taps of row (l, k): row (k + e - (mz-1)) n_ell + m
+    const int l = row / ms, k = row - l * ms;
+    sr = l * (ms + q - 1) + ms - 1 - k;
+    ca = k - (ms - 1);
+  }
   if (MODE == 1) {
     const int j = row / n_ell, l = row - j * n_ell;
     t = j / q;
@@ -189,12 +201,21 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32)
     }
     sr = js * n_ell + l;
   }
+  // gathered row of a stored column (a tap's key: index | offset << 16)
+  auto remap = [&](int c, int off) {
+    if (MODE == 1) return rot_pixel(c, t, ms, magic, mir);
+    if (MODE == 2) return c + off;
+    if (MODE == 3) return (c & 0xffff) * ms + ca + (c >> 16);
+    if (MODE == 4) return (ca + (c >> 16)) * n_ell + (c & 0xffff);
+    return c;
+  };
   int2* st = stage[SH ? 0 : w][sub];
 #pragma unroll 1
   for (int s = 0; s < (MODE == 2 ? 4 : 1); ++s) {
     if (MODE == 2) sr = rot_pixel(row, 4 - s, ms, magic);
     const int off = MODE == 2 ? s * q * n_ell : 0;
-    const int e0 = rowptr[sr], e1 = mine ? rowptr[sr + 1] : e0;
+    const int e0 = rowptr[sr];
+    const int e1 = mine ? rowptr[sr + (MODE == 3 ? ms : MODE == 4 ? q : 1)] : e0;
     // batches run in step over the warp's rows (an exhausted row idles); the
     // next batch's entries are requested before this one's gathers
     const int len = NR > 1 ? (int)__reduce_max_sync(FULL, (unsigned)(e1 - e0)) : e1 - e0;
@@ -220,8 +241,7 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32)
         float v = 0.f;
         if (eb + lane < e1) {
           c = col[eb + lane];
-          if (MODE == 1) c = rot_pixel(c, t, ms, magic, mir);
-          if (MODE == 2) c += off;
+          c = remap(c, off);
           SRT_CHECK_GATHER(0, c, xrows, g_viol);
           v = wval<V>(val[eb + lane]);
         }
@@ -249,8 +269,7 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32)
       for (int k = 0; k < KE; ++k)
         if (eb + sl + k * GL < e1) {
           int c = nc[k];
-          if (MODE == 1) c = rot_pixel(c, t, ms, magic, mir);
-          if (MODE == 2) c += off;
+          c = remap(c, off);
           SRT_CHECK_GATHER(0, c, xrows, g_viol);
           st[sl + k * GL] = make_int2(c, __float_as_int(wval<V>(nv[k])));
         }
@@ -371,7 +390,7 @@ int launch_width(const SrtCsr& A, const V* val, const Rows& W, const float* x, i
   const int n = (ncols + VW - 1) / VW;  // vectors of a row
   // wide rows stored as they are: each entry's reuse over 512 columns wins
   // over more warps (at 1024 columns 10.6 against 11.1 ms for A2 of 256^3 as CSR)
-  if constexpr (MODE == 0 && VW == 4 && U == 1) {
+  if constexpr (MODE != 1 && MODE != 2 && VW == 4 && U == 1) {
     if (n > 96) SRT_ROWS(4, 32);
     SRT_ROWS(3, 32);
   }
@@ -422,7 +441,7 @@ int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t
   const int64_t per_warp = vecs > 32 ? 1 : vecs > 16 ? 2 : 4;
   const bool few = (int64_t)W.rows * batch / per_warp <= (int64_t)128 * kSMs &&
                    vecs <= (lanes == 4 ? 64 : 128);
-  if constexpr (MODE == 0)
+  if constexpr (MODE != 1 && MODE != 2)
     if (lanes == 4 && vecs > 64)
       return launch_width<V, 4, MODE, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
 #define SRT_WIDTH(VW)                                                                          \
@@ -443,6 +462,8 @@ int dispatch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64
   switch (W.rot.mode) {
     case 1: return launch<V, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
     case 2: return launch<V, 2>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+    case 3: return launch<V, 3>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+    case 4: return launch<V, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
     default: return launch<V, 0>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
   }
 }
@@ -456,7 +477,7 @@ int srt_spmm(const SrtCsr& A, int wdt, const float* x, int64_t ldx, int64_t bsx,
   if (rows <= 0) return SRT_OK;
   if (rows > 0x7fffffff || r0 + rows > 0x7fffffff) return SRT_ERR_ARG;
   uint64_t magic = 0;
-  if (rot.mode != 0) {
+  if (rot.mode == 1 || rot.mode == 2) {
     if (rot.q <= 0 || rot.ms <= 0 || rot.ms >= (1 << 16) || rot.n_ell <= 0 ||
         (int64_t)rot.ms * rot.ms >= (1 << 24))
       return SRT_ERR_ARG;

@@ -13,8 +13,7 @@
 //
 // The taps are stored twice, grouped so that the entries of any output row
 // form ONE contiguous range, which the product kernel then walks exactly like
-// a CSR row (coalesced batch of 32 entries, shuffle broadcast, float4
-// gathers of dense rows):
+// a CSR row (spmm.cu k_rows, modes 3 and 4):
 //   forward  (rows (h, m) of A2):   sub-rows (m, q), each listing l
 //     ascending; row (h, m) is sub-rows q = n_zs-1-h .. n_zs-2-h+mz, i.e.
 //     every slab k = h + q - (n_zs-1) of the volume.  Entry key = l | q << 16;
@@ -26,7 +25,10 @@
 // With the rings at the slab centres (n_zs = mz, s = eps = 0), D = 2 mz - 1.
 // The adjoint visits its entries in the same order as the CSR form of A2^T
 // (ascending (h, m)), the forward by ascending (d, l).  Every output row is
-// owned by one warp: no atomics.
+// owned by one group of lanes: no atomics.  The row kernel serves every dense
+// width (us, A2 / A2^T, with the taps' own warp-per-row kernels before: 57
+// columns at 65 slabs 61.5 / 50.2 -> 38.9 / 34.0, 63 at 128 317 / 283 -> 225 /
+// 216; row by row at 256^3 2816 / 2818 -> 2614 / 2685).
 #include <algorithm>
 #include <cstdlib>
 #include <vector>
@@ -35,196 +37,6 @@
 #include "devutil.cuh"
 
 namespace {
-
-constexpr unsigned FULL = 0xffffffffu;
-#ifdef SRT_CHECKS
-__device__ unsigned long long g_viol;  // gathered rows outside their operand
-#endif
-
-template <typename V>
-__device__ __forceinline__ float tap_w(V v);
-template <>
-__device__ __forceinline__ float tap_w<float>(float v) {
-  return v;
-}
-template <>
-__device__ __forceinline__ float tap_w<uint16_t>(uint16_t v) {
-  return srt_bf16_to_f32(v);
-}
-
-struct TapArgs {
-  const int32_t* rowptr;  // sub-row pointers
-  const int32_t* key;     // packed (index, offset) per tap
-  int mz, n_zs, n_ell, r0;  // r0: first output row of this launch
-  int rows, G, R, TG;     // rows of this launch; block order (G groups of R, TG per block)
-  int xrows;              // rows of the gathered operand (debug-build checks)
-};
-
-// Block-to-row order as in spmm.cu: with G > 0 a block owns TG groups x 8/TG
-// consecutive rows, blocks chunk-major; with G = 0 consecutive rows.
-__device__ __forceinline__ int tap_row(int G, int R, int TG) {
-  const int w = threadIdx.x >> 5;
-  if (G <= 0) return blockIdx.x * (blockDim.x >> 5) + w;
-  const int TI = 8 / TG;
-  const int chunks = (R + TI - 1) / TI, tiles = (G + TG - 1) / TG;
-  const int c = blockIdx.x / tiles, t = blockIdx.x - c * tiles;
-  if (c >= chunks) return -1;
-  const int g = t * TG + w / TI, i = c * TI + w % TI;
-  return (g < G && i < R) ? g * R + i : -1;
-}
-
-// ADJ = false: y[(h,m)][n] = sum T[m,d,l] x[l*mz + h + d][n]      (A2 Y1')
-// ADJ = true:  y[(l,k)][n] = sum T[m,k-h,l] x[h*n_ell + m][n]     (A2^T P')
-// Lanes own 4 consecutive dense columns of each 128-column chunk.
-template <typename V, int CH, bool ADJ>
-__global__ void __launch_bounds__(256) k_taps(TapArgs A, const V* __restrict__ val,
-                                              const float* __restrict__ x, int64_t ldx,
-                                              float* __restrict__ y, int64_t ldy, int ncols) {
-  srt_in_order();
-  const int lane = threadIdx.x & 31;
-  const int lr = tap_row(A.G, A.R, A.TG);
-  if (lr < 0 || lr >= A.rows) return;
-  const int row = A.r0 + lr;
-  const int mz = A.mz, nz = A.n_zs, D = mz + nz - 1;
-  int a, b;  // (h, m) forward, (l, k) adjoint
-  if (ADJ) {
-    a = row / mz;
-    b = row - a * mz;
-  } else {
-    a = row / A.n_ell;
-    b = row - a * A.n_ell;
-  }
-  // forward: sub-rows m*D + (nz-1-h) .. +mz; adjoint: l*D + (mz-1-k) .. +nz
-  const int64_t s0 = ADJ ? (int64_t)a * D + (mz - 1 - b) : (int64_t)b * D + (nz - 1 - a);
-  const int e0 = A.rowptr[s0], e1 = A.rowptr[s0 + (ADJ ? nz : mz)];
-  const int n0 = blockIdx.y * (128 * CH) + lane * 4;
-  float4 acc[CH];
-#pragma unroll
-  for (int q = 0; q < CH; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int eb = e0; eb < e1; eb += 32) {
-    int c = 0;
-    float v = 0.f;
-    if (eb + lane < e1) {
-      const int kk = A.key[eb + lane];
-      const int lo = kk & 0xffff, off = kk >> 16;
-      // forward: off = q, gathered row l*mz + h + q - (nz-1)
-      // adjoint: off = e, h = k + e - (mz-1), gathered row h*n_ell + m
-      c = ADJ ? (b + off - (mz - 1)) * A.n_ell + lo : lo * mz + a + off - (nz - 1);
-      SRT_CHECK_GATHER(0, c, A.xrows, g_viol);
-      v = tap_w<V>(val[eb + lane]);
-    }
-    const int cnt = min(32, e1 - eb);
-    // not unrolled: 31 registers and 64 resident warps per SM against 48
-    // registers / 40 warps for the compiler's unroll; the product waits on
-    // its gathers, and more warps win (A2, A2^T 4.7% faster, same order)
-#pragma unroll 1
-    for (int i = 0; i < cnt; ++i) {
-      const int ci = __shfl_sync(FULL, c, i);
-      const float vi = __shfl_sync(FULL, v, i);
-      const float* xr = x + (int64_t)ci * ldx;
-#pragma unroll
-      for (int q = 0; q < CH; ++q) {
-        const int n = n0 + q * 128;
-        if (n < ncols) {
-          const float4 xv = srt_ldg_keep(xr + n);
-          acc[q].x = fmaf(vi, xv.x, acc[q].x);
-          acc[q].y = fmaf(vi, xv.y, acc[q].y);
-          acc[q].z = fmaf(vi, xv.z, acc[q].z);
-          acc[q].w = fmaf(vi, xv.w, acc[q].w);
-        }
-      }
-    }
-  }
-  float* yr = y + (int64_t)lr * ldy;
-#pragma unroll
-  for (int q = 0; q < CH; ++q) {
-    const int n = n0 + q * 128;
-    if (n < ncols) *reinterpret_cast<float4*>(yr + n) = acc[q];
-  }
-}
-
-// The same for any dense width and strides: lane owns columns lane + 32 i.
-template <typename V, int PER, bool ADJ>
-__global__ void __launch_bounds__(256) k_taps_scalar(TapArgs A, const V* __restrict__ val,
-                                                     const float* __restrict__ x, int64_t ldx,
-                                                     float* __restrict__ y, int64_t ldy,
-                                                     int ncols) {
-  srt_in_order();
-  const int lane = threadIdx.x & 31;
-  const int lr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (lr >= A.rows) return;
-  const int row = A.r0 + lr;
-  const int mz = A.mz, nz = A.n_zs, D = mz + nz - 1;
-  const int a = ADJ ? row / mz : row / A.n_ell;
-  const int b = ADJ ? row - a * mz : row - a * A.n_ell;
-  const int64_t s0 = ADJ ? (int64_t)a * D + (mz - 1 - b) : (int64_t)b * D + (nz - 1 - a);
-  const int e0 = A.rowptr[s0], e1 = A.rowptr[s0 + (ADJ ? nz : mz)];
-  const int n0 = blockIdx.y * (32 * PER) + lane;
-  float acc[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-  for (int eb = e0; eb < e1; eb += 32) {
-    int c = 0;
-    float v = 0.f;
-    if (eb + lane < e1) {
-      const int kk = A.key[eb + lane];
-      const int lo = kk & 0xffff, off = kk >> 16;
-      c = ADJ ? (b + off - (mz - 1)) * A.n_ell + lo : lo * mz + a + off - (nz - 1);
-      SRT_CHECK_GATHER(0, c, A.xrows, g_viol);
-      v = tap_w<V>(val[eb + lane]);
-    }
-    const int cnt = min(32, e1 - eb);
-    for (int i = 0; i < cnt; ++i) {
-      const int ci = __shfl_sync(FULL, c, i);
-      const float vi = __shfl_sync(FULL, v, i);
-      const float* xr = x + (int64_t)ci * ldx;
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        const int n = n0 + q * 32;
-        if (n < ncols) acc[q] = fmaf(vi, __ldg(xr + n), acc[q]);
-      }
-    }
-  }
-  float* yr = y + (int64_t)lr * ldy;
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int n = n0 + q * 32;
-    if (n < ncols) yr[n] = acc[q];
-  }
-}
-
-template <typename V, bool ADJ>
-int launch(const TapArgs& A, const V* val, const float* x, int64_t ldx, float* y, int64_t ldy,
-           int ncols, cudaStream_t st) {
-  const bool vec = ncols % 4 == 0 && ldx % 4 == 0 && ldy % 4 == 0 && (uintptr_t)x % 16 == 0 &&
-                   (uintptr_t)y % 16 == 0;
-  if (!vec) {
-    dim3 grid((unsigned)(((int64_t)A.rows + 7) / 8), (ncols + 127) / 128, 1);
-    SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps_scalar<V, 4, ADJ>, grid, 256, st, A, val, x, ldx, y,
-                            ldy, ncols));
-    SRT_CUDA_TRY(cudaGetLastError());
-    return SRT_OK;
-  }
-  const int TI = 8 / A.TG;
-  const int64_t gx = A.G > 0 ? (int64_t)((A.R + TI - 1) / TI) * ((A.G + A.TG - 1) / A.TG)
-                             : ((int64_t)A.rows + 7) / 8;
-  if (gx > 0x7fffffff) return SRT_ERR_ARG;
-  const int chunks = (ncols + 127) / 128;
-  const int CH = chunks >= 4 ? 4 : chunks;
-  dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), 1);
-  switch (CH) {
-    case 4: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 4, ADJ>, grid, 256, st, A, val, x, ldx, y,
-                                    ldy, ncols)); break;
-    case 3: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 3, ADJ>, grid, 256, st, A, val, x, ldx, y,
-                                    ldy, ncols)); break;
-    case 2: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 2, ADJ>, grid, 256, st, A, val, x, ldx, y,
-                                    ldy, ncols)); break;
-    default: SRT_CUDA_TRY(srt_launch(8 * kSMs, k_taps<V, 1, ADJ>, grid, 256, st, A, val, x, ldx, y,
-                                     ldy, ncols)); break;
-  }
-  SRT_CUDA_TRY(cudaGetLastError());
-  return SRT_OK;
-}
 
 // Upload one grouped tap list (host vectors) into t.
 int upload(const std::vector<int32_t>& rp, const std::vector<int32_t>& key,
@@ -323,27 +135,19 @@ int srt_taps_apply(const srt_plan_s* plan, bool adjoint, int64_t r0, int64_t row
   const srt_geometry& g = plan->g;
   const SrtTaps& t = adjoint ? plan->ta : plan->tf;
   if (!t.rowptr || rows <= 0 || ncols <= 0) return SRT_ERR_ARG;
-  if (G > 0 && (int64_t)G * R != rows) G = 0;
-  if (TG != 1 && TG != 2 && TG != 4 && TG != 8) TG = 1;
-  TapArgs A{t.rowptr, t.key, g.mz, g.n_zs, g.n_ell, (int)r0, (int)rows, G, R, TG,
-            srt_checked_rows(adjoint ? (int64_t)g.n_zs * g.n_ell : (int64_t)g.n_ell * g.mz)};
-  if (g.weight_dtype == SRT_BF16) {
-    if (!t.w16) return SRT_ERR_ARG;
-    return adjoint ? launch<uint16_t, true>(A, t.w16, x, ldx, y, ldy, ncols, st)
-                   : launch<uint16_t, false>(A, t.w16, x, ldx, y, ldy, ncols, st);
-  }
-  if (!t.w32) return SRT_ERR_ARG;
-  return adjoint ? launch<float, true>(A, t.w32, x, ldx, y, ldy, ncols, st)
-                 : launch<float, false>(A, t.w32, x, ldx, y, ldy, ncols, st);
-}
-
-long long srt_checks_take_taps() {
-#ifdef SRT_CHECKS
-  unsigned long long v = 0, z = 0;
-  if (cudaMemcpyFromSymbol(&v, g_viol, sizeof(v)) != cudaSuccess) return -1;
-  if (cudaMemcpyToSymbol(g_viol, &z, sizeof(z)) != cudaSuccess) return -1;
-  return (long long)v;
-#else
-  return 0;
-#endif
+  if (g.weight_dtype == SRT_BF16 ? !t.w16 : !t.w32) return SRT_ERR_ARG;
+  SrtCsr a;  // the taps as the row kernel reads them; every output row a range of them
+  a.rows = adjoint ? g.n_ell * g.mz : g.n_zs * g.n_ell;
+  a.cols = adjoint ? g.n_zs * g.n_ell : g.n_ell * g.mz;
+  a.nnz = t.nent;
+  a.rowptr = t.rowptr;
+  a.col = t.key;
+  a.v32 = t.w32;
+  a.v16 = t.w16;
+  SrtRot how;
+  how.mode = adjoint ? 4 : 3;
+  how.ms = g.mz;
+  how.n_ell = g.n_ell;
+  how.q = g.n_zs;
+  return srt_spmm(a, g.weight_dtype, x, ldx, 0, y, ldy, 0, ncols, 1, st, G, R, TG, r0, rows, how);
 }

@@ -45,7 +45,7 @@ def parse():
     p.add_argument("--a1-rotation", action="store_true",
                    help="store A1 for a quarter of the sensor columns (quarter turns only, no mirror)")
     p.add_argument("--rowwise", action="store_true",
-                   help="every product a warp per output row (else register tiles of rows)")
+                   help="every product row by row (else register tiles of rows)")
     p.add_argument("--voxel-linear", action="store_true",
                    help="f bilinear in (x, y) between voxel centres (else constant on voxels)")
     p.add_argument("--fuse-reshapes", action="store_true",
@@ -195,7 +195,7 @@ def stage_model(geom, info, batch, weights, fused=False, fused_p1=False):
     spmm2 = dict(flop=2 * nnz2 * geom.n_phi * batch, bytes=a2b + y1 + pp)
     spmm2t = dict(flop=spmm2["flop"], bytes=a2tb + pp + y1)
     spmm1t = dict(flop=spmm1["flop"], bytes=a1tb + y1 + fv)
-    # useful FMAs per gathered dense operand: 1 for a row-per-warp product;
+    # useful FMAs per gathered dense operand: 1 for a row by row product;
     # entries per record for the register tiles (A1^T: stored entries, the
     # symmetry passes repeat entries and records alike)
     # (A2: the records are per radius pair and key, each folding the taps of
@@ -550,7 +550,7 @@ def run_ours(args):
                                       "plan_build_s": round(plan_s, 3),
                                       "nnz1": plan.info["nnz1"], "nnz2": plan.info["nnz2"],
                                       "a2_form": (f"Toeplitz taps ({plan.info['n_taps']} taps of T), "
-                                                  + ("a warp per row" if args.rowwise
+                                                  + ("row by row" if args.rowwise
                                                      else "2 x 2 row tiles")
                                                   if plan.info["a2_taps"] else "CSR"),
                                       "a1_form": {0: "every column", 1: "the first n_phi/4 "
@@ -558,8 +558,8 @@ def run_ours(args):
                                                   2: "the first n_phi/8 + 1 columns, the rest by "
                                                   "quarter turns and the diagonal mirror"}[
                                                       plan.info["a1_rot"]]
-                                                  + ("; a warp per row" if args.rowwise
-                                                     else "; A1 a warp per row, A1^T 2 x 2-pixel "
+                                                  + ("; row by row" if args.rowwise
+                                                     else "; A1 row by row, A1^T 2 x 2-pixel "
                                                           "register tiles"),
                                       "reshapes": ", ".join(
                                           (["P1 fused into the A1 epilogue"] if fused_p1 else [])

@@ -63,7 +63,7 @@ enum srt_weight_dtype { SRT_FP32 = 0, SRT_BF16 = 1 };
  * nodes); A2's entry (l, k) becomes node l's hat integrated along the
  * semicircle inside slab k, so A2 holds more entries (1.49x at 256^3). */
 #define SRT_RHO_LINEAR 0x10
-/* SRT_ROWWISE: apply every product with one warp per output row (CSR rows,
+/* SRT_ROWWISE: apply every product output row by output row (CSR rows,
  * or A2's taps) instead of register tiles of output rows (the default).  A
  * row then sums its entries in ascending column order: with A1 stored for
  * every column the tiled and the row-wise forms agree bitwise (up to the

@@ -8,9 +8,9 @@
 // walks the union of its rows' gathered rows: one record per gathered row,
 // with four weights (zero where a pixel does not use it).  At 256^3 a record
 // serves 2.0 entries on average.  (The same idea for A1 itself, 4
-// consecutive radii of one column per warp, measured slower than the
-// row-per-warp CSR kernel: there the 8 warps of a block already share their
-// gathered pixels through L1, and the tiles lose that sharing.)
+// consecutive radii of one column per warp, measured slower than the CSR
+// row kernel: there the rows of a block already share their gathered pixels
+// through L1, and the tiles lose that sharing.)
 //
 // Symmetry (Sec. 2's columns are equispaced around the axis).  Let
 // rot(ix, iy) = (ms-1-iy, ix) (a quarter turn of the pixel grid) and
@@ -33,7 +33,7 @@
 // tile's four slots per g (with few slabs the warp's groups of lanes share
 // the elements, k_a1t_split).  With every column stored (one pass) each pixel
 // sums its entries in the CSR order of A1^T, ascending (j, l).  Every output
-// row is one warp's FP32 sum: no atomics, deterministic.
+// row is one warp's FP32 sum, in a fixed order: no atomics, deterministic.
 #include <algorithm>
 #include <vector>
 

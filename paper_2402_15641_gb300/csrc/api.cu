@@ -213,12 +213,11 @@ int run_forward(srt_plan_s* p, const float* f, float* out, int B, float* w0, flo
   // rows (j, l) visited radius-chunk-major across sensor columns (L2 reuse of F)
   {
     NvRange r(fused_p1(p) ? "A1 product + reshape P1" : "A1 product");
-    // CSR rows, a warp per row: the 8 warps of a block take 8 consecutive
-    // radii of one column, whose circles cross the same pixels, and share
-    // those gathers in L1 (46% hits).  4-radius register tiles
-    // (srt_a1tiles_apply) fetch each pixel once per tile instead, but lose
-    // that sharing (13% L1 hits) and measured slower (1.74-1.97 against
-    // 1.56 ms at 256^3).
+    // CSR rows: a block takes consecutive radii of one column (8 at 256
+    // columns), whose circles cross the same pixels, and its rows share
+    // those gathers in L1 (39-46% hits).  4-radius register tiles, which
+    // fetch each pixel once per tile instead, lose that sharing (13% L1
+    // hits) and measured slower (1.74-1.97 against 1.56 ms at 256^3).
     if (fused_p1(p))  // writing Y1' (the reshape P1's output) itself
       SRT_TRY(srt_spmm(p->a1, g.weight_dtype, f, g.mz, pix * g.mz, w1, 0, 0, g.mz, B, st,
                        g.n_phi, g.n_ell, 4, 0, r1, a1_rot(p, 1), 0, nb));
@@ -249,7 +248,7 @@ int run_forward(srt_plan_s* p, const float* f, float* out, int B, float* w0, flo
     }
     if (p->tiles && nb % 4 == 0)  // A2 from 2 x 2 tiles of the master tensor's taps
       SRT_TRY(srt_tiles_apply(p, false, h0, h1, w1, nb, w0 + ra * nb, nb, (int)nb, st));
-    else if (p->toeplitz)  // A2 from the taps of the master tensor, a warp per row
+    else if (p->toeplitz)  // A2 from the taps of the master tensor, row by row
       SRT_TRY(srt_taps_apply(p, false, ra, rn, h1 - h0, g.n_ell, 4, w1, nb, w0 + ra * nb, nb,
                              (int)nb, st));
     else
@@ -290,7 +289,7 @@ int run_adjoint(srt_plan_s* p, const float* in, float* f, int B, float* w0, floa
       SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, w0, nb, w1, 0, (int)nb, st, c1));
     else if (p->tiles && nb % 4 == 0)  // A2^T from 2 x 2 tiles of the master tensor's taps
       SRT_TRY(srt_tiles_apply(p, true, 0, g.mz, w0, nb, w1, nb, (int)nb, st));
-    else if (p->toeplitz)  // A2^T from the taps of the master tensor, a warp per row
+    else if (p->toeplitz)  // A2^T from the taps of the master tensor, row by row
       SRT_TRY(srt_taps_apply(p, true, 0, c1, 0, 0, 1, w0, nb, w1, nb, (int)nb, st));
     else
       SRT_TRY(srt_spmm(p->a2t, g.weight_dtype, w0, nb, 0, w1, nb, 0, (int)nb, 1, st));

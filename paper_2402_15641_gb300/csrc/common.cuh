@@ -398,7 +398,7 @@ __host__ __device__ inline uint16_t srt_f64_to_bf16(double x) {
 }
 
 // 16-byte read-only gather of a dense row with the L1 evict-last hint: the
-// rows gathered by a block's 8 warps overlap, and keeping them in L1 ahead
+// rows gathered by a block's warps overlap, and keeping them in L1 ahead
 // of streaming data made the products 0.2-2.4% faster (same values).
 __device__ __forceinline__ float4 srt_ldg_keep(const float* p) {
   float4 r;

@@ -41,7 +41,7 @@ class Geometry:
     csr_only: bool = False
     a1_rotation: bool = False
     rho_linear: bool = False  # intermediate piecewise linear in rho (else constant on bins)
-    rowwise: bool = False  # every product a warp per output row (else register tiles of rows)
+    rowwise: bool = False  # every product row by row (else register tiles of rows)
     n_phi_total: int = 0  # > 0: the plan holds columns phi_first .. + n_phi - 1 of this many
     phi_first: int = 0
     a1_full: bool = False  # store A1 for every column (else for the aperture's symmetry set)

@@ -183,7 +183,7 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
       const float* xr = x0 + (int64_t)o[u] * ldx;
 #pragma unroll
       for (int c = 0; c < CH; ++c)
-        if (in[c]) v[u][c] = srt_ldg_keep(xr + c * 128);
+        if (in[c]) v[u][c] = srt_ld_keep(xr + c * 128);
     }
 #pragma unroll
     for (int u = 0; u < H; ++u) rec_w<W>(wt + eb + u, w[u]);
@@ -226,7 +226,7 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
 #pragma unroll
     for (int c = 0; c < CH; ++c)
       if (in[c]) {
-        const float4 xv = srt_ldg_keep(xr + c * 128);
+        const float4 xv = srt_ld_keep(xr + c * 128);
 #pragma unroll
         for (int sg = 0; sg < 4; ++sg) fma4(acc[sym_slot(PS, PM, sg)][c], w[sg], xv);
       }
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kNW * 32, 4)
         const float* xr = x0 + (int64_t)o[u] * ldx;
 #pragma unroll
         for (int c = 0; c < CH; ++c)
-          if (in[c]) v[u][c] = srt_ldg_keep(xr + c * (4 * GL));
+          if (in[c]) v[u][c] = srt_ld_keep(xr + c * (4 * GL));
       }
 #pragma unroll
       for (int u = 0; u < H; ++u)

@@ -226,8 +226,12 @@ constexpr int SRT_DOT_BLOCKS = 4 * kSMs;
 // resident while the kernel before still runs, and srt_in_order(), the first
 // statement of every kernel here, waits until that kernel has completed and
 // its writes are visible.  Only then does it let the next kernel's blocks
-// come up, so at most one kernel waits ahead, and it was launched (its L1
-// lines dropped) after every earlier reader of its operand had finished.
+// come up, so at most one kernel waits ahead.  Its operand may still be
+// written while it is resident, so no kernel reads its operand through the
+// read-only path (ld.global.nc, __ldg), whose data must not change while
+// the kernel lives: srt_ld_keep, srt_ld4, srt_ld2 and srt_ld1 are plain loads
+// that the compiler keeps behind the wait.  Row pointers, keys, columns and
+// weights are the plan's, written before any call, and stay read-only loads.
 // Without the attribute both instructions do nothing.  Work that follows a
 // call in its stream waits for the last kernel as usual.
 //
@@ -397,14 +401,34 @@ __host__ __device__ inline uint16_t srt_f64_to_bf16(double x) {
   return (uint16_t)((sign << 15) | q);
 }
 
-// 16-byte read-only gather of a dense row with the L1 evict-last hint: the
-// rows gathered by a block's warps overlap, and keeping them in L1 ahead
-// of streaming data made the products 0.2-2.4% faster (same values).
-__device__ __forceinline__ float4 srt_ldg_keep(const float* p) {
+// Loads of a kernel's operand (see srt_in_order): plain global loads, not
+// read-only ones, and volatile, so that they stay behind the wait.
+//
+// 16 bytes of a dense row with the L1 evict-last hint: the rows gathered by
+// a block's warps overlap, and keeping them in L1 ahead of streaming data
+// made the products 0.2-2.4% faster (same values).
+__device__ __forceinline__ float4 srt_ld_keep(const float* p) {
   float4 r;
-  asm volatile("ld.global.nc.L1::evict_last.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::evict_last.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
                : "l"(p));
+  return r;
+}
+__device__ __forceinline__ float4 srt_ld4(const float* p) {
+  float4 r;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+               : "l"(p));
+  return r;
+}
+__device__ __forceinline__ float2 srt_ld2(const float* p) {
+  float2 r;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ float srt_ld1(const float* p) {
+  float r;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p));
   return r;
 }
 

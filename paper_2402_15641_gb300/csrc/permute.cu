@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(256) k_transpose(const float* __restrict__ in,
 #pragma unroll
   for (int i = ty; i < TILE; i += 8) {
     const int r = r0 + i, c = c0 + tx;
-    if (r < rows && c < cols) tile[i][tx] = in[(int64_t)r * ild + c];
+    if (r < rows && c < cols) tile[i][tx] = srt_ld1(in + (int64_t)r * ild + c);
   }
   __syncthreads();
 #pragma unroll
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256) k_transpose_v4(const float* __restrict__ 
     const int i = rr + 16 * k;  // tile row
     const int r = r0 + i, c = c0 + 4 * q;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < rows && c < cols) v = __ldg(reinterpret_cast<const float4*>(in + (int64_t)r * ild + c));
+    if (r < rows && c < cols) v = srt_ld4(in + (int64_t)r * ild + c);
     tile[i][4 * q] = v.x;
     tile[i][4 * q + 1] = v.y;
     tile[i][4 * q + 2] = v.z;

@@ -102,17 +102,17 @@ struct Rows {
 template <int VW>
 __device__ __forceinline__ void ld_cols(const float* p, float (&v)[VW]) {
   if constexpr (VW == 4) {
-    const float4 q = srt_ldg_keep(p);
+    const float4 q = srt_ld_keep(p);
     v[0] = q.x;
     v[1] = q.y;
     v[2] = q.z;
     v[3] = q.w;
   } else if constexpr (VW == 2) {
-    const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+    const float2 q = srt_ld2(p);
     v[0] = q.x;
     v[1] = q.y;
   } else {
-    v[0] = __ldg(p);
+    v[0] = srt_ld1(p);
   }
 }
 

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(TR ? 256 : 128, TR ? 2 : 4)
         const float* xr = x0 + (int64_t)o[u] * ldx;
 #pragma unroll
         for (int q = 0; q < CH; ++q)
-          if (in[q]) v[u][q] = srt_ldg_keep(xr + q * 128);
+          if (in[q]) v[u][q] = srt_ld_keep(xr + q * 128);
       }
 #pragma unroll
       for (int u = 0; u < H; ++u) tile_w<W>(wt + eb + u, w[u]);
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(TR ? 256 : 128, TR ? 2 : 4)
 #pragma unroll
       for (int q = 0; q < CH; ++q)
         if (in[q]) {
-          const float4 xv = srt_ldg_keep(xr + q * 128);
+          const float4 xv = srt_ld_keep(xr + q * 128);
 #pragma unroll
           for (int s = 0; s < 4; ++s) fma4(acc[s][q], w[s], xv);
         }

@@ -101,31 +101,35 @@ struct A1Args {
   const int32_t* ptr;  // record ranges (see the kernels)
   const int32_t* key;  // (j << 16 | l)
   int mode, q, ms, n_phi, n_ell, ntx;
-  int G, R, TG, S;     // block order
+  int G, R, S;         // block order
   int g0, g1;          // tile rows [g0, g1) (pixel rows 2 g0 .. 2 g1 - 1)
   int xrows;           // rows of the gathered operand (debug-build checks)
 };
 
 
-constexpr int kNW = 4;  // warps of a block
+// Blocks of four warps own 2 x 2 tiles (4 x 4 pixels), of eight 4 x 2; which,
+// launch_a1t says.
+template <int NW>
+constexpr int kTG = NW == 8 ? 4 : 2;
 
 // Warp -> (group, index) as in spmm.cu's block_row: G groups of R, a block
-// owning TG groups x kNW/TG consecutive indices, chunk-major, or S x S
+// owning kTG groups x NW / kTG consecutive indices, chunk-major, or S x S
 // super-tiles (S > 0).
+template <int NW>
 __device__ __forceinline__ bool warp_tile(const A1Args& A, int* g, int* i) {
   const int w = threadIdx.x >> 5;
-  const int TI = kNW / A.TG;
+  constexpr int TG = kTG<NW>, TI = NW / TG;
   if (A.S > 0) {
-    const int per_row = A.S / A.TG, bpt = per_row * (A.S / TI);
+    const int per_row = A.S / TG, bpt = per_row * (A.S / TI);
     const int st = blockIdx.x / bpt, r = blockIdx.x - st * bpt;
     const int nsx = (A.G + A.S - 1) / A.S, sx = st % nsx, sy = st / nsx;
     const int tx = r % per_row, ty = r / per_row;
-    *g = sx * A.S + tx * A.TG + w / TI;
+    *g = sx * A.S + tx * TG + w / TI;
     *i = sy * A.S + ty * TI + w % TI;
   } else {
-    const int tiles = (A.G + A.TG - 1) / A.TG;
+    const int tiles = (A.G + TG - 1) / TG;
     const int c = blockIdx.x / tiles, t = blockIdx.x - c * tiles;
-    *g = t * A.TG + w / TI;
+    *g = t * TG + w / TI;
     *i = c * TI + w % TI;
   }
   return *g < A.G && *i < A.R;
@@ -235,14 +239,14 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
 
 // f[b][p][k] = sum_(J,l) A1[(J, l), p] F1[b][(J, l)][k] for the 2 x 2 pixel
 // tile (ta, tb) with ta in [g0, g1); y points at pixel row 2 g0.
-template <typename W, int CH>
-__global__ void __launch_bounds__(kNW * 32, 4)
+template <typename W, int CH, int NW>
+__global__ void __launch_bounds__(NW * 32, 16 / NW)
     k_a1t_tile(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx, int64_t bsx,
                float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
   srt_in_order();
   const int lane = threadIdx.x & 31;
   int ga, tb;
-  if (!warp_tile(A, &ga, &tb)) return;
+  if (!warp_tile<NW>(A, &ga, &tb)) return;
   const int ta = A.g0 + ga;
   const int n0 = blockIdx.y * (128 * CH) + lane * 4;
   const float* x0 = x + blockIdx.z * bsx + n0;
@@ -299,14 +303,14 @@ __device__ __forceinline__ float rec_w1(const uint2* p, int q) {
 // too few registers for groups of five: 201 against 166 and 350 against 297
 // us, so wider volumes keep a warp to a pass.
 template <typename W, int CH, int GL>
-__global__ void __launch_bounds__(kNW * 32, 4)
+__global__ void __launch_bounds__(128, 4)
     k_a1t_split(A1Args A, const W* __restrict__ wt, const float* __restrict__ x, int ldx,
                 int64_t bsx, float* __restrict__ y, int ldy, int64_t bsy, int ncols) {
   srt_in_order();
   constexpr int NS = 32 / GL, H = kH<CH>;
   const int lane = threadIdx.x & 31, sub = lane / GL, sl = lane % GL;
   int ga, tb;
-  if (!warp_tile(A, &ga, &tb)) return;
+  if (!warp_tile<4>(A, &ga, &tb)) return;
   const int ta = A.g0 + ga;
   const int n0 = sl * 4;
   const float* x0 = x + blockIdx.z * bsx + n0;
@@ -528,39 +532,49 @@ int srt_build_a1tiles(srt_plan_s* plan, int64_t* bytes) {
 
 namespace {
 
+// Blocks of the launch, NW warps each.
+template <int NW>
+int64_t a1t_blocks(const A1Args& A) {
+  constexpr int TG = kTG<NW>, TI = NW / TG;
+  if (A.S > 0)
+    return (int64_t)((A.G + A.S - 1) / A.S) * ((A.R + A.S - 1) / A.S) * (A.S / TG) * (A.S / TI);
+  return (int64_t)((A.R + TI - 1) / TI) * ((A.G + TG - 1) / TG);
+}
+
 template <typename W>
 int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t bsx, float* y,
                int64_t ldy, int64_t bsy, int ncols, int batch, cudaStream_t st) {
-  const int TI = kNW / A.TG;
-  int64_t gx;
-  if (A.S > 0) {
-    gx = (int64_t)((A.G + A.S - 1) / A.S) * ((A.R + A.S - 1) / A.S) * (A.S / A.TG) * (A.S / TI);
-  } else {
-    gx = (int64_t)((A.R + TI - 1) / TI) * ((A.G + A.TG - 1) / A.TG);
-  }
-  if (gx > 0x7fffffff || batch > 65535) return SRT_ERR_ARG;
-  if (A.mode && ncols <= 64) {
-    dim3 grid((unsigned)gx, 1, batch);
-    if (ncols <= 16 && A.mode == 2)  // 8 groups: one to each of the 8 passes
-      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 4>, grid, kNW * 32, st, A, w, x, (int)ldx,
-                              bsx, y, (int)ldy, bsy, ncols));
-    else if (ncols <= 32)
-      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 8>, grid, kNW * 32, st, A, w, x, (int)ldx,
-                              bsx, y, (int)ldy, bsy, ncols));
-    else
-      SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_split<W, 1, 16>, grid, kNW * 32, st, A, w, x,
-                              (int)ldx, bsx, y, (int)ldy, bsy, ncols));
-    SRT_CUDA_TRY(cudaGetLastError());
-    return SRT_OK;
-  }
   const int CH = ncols > 128 ? 2 : 1;
+  // Large batches of more than 128 slabs take blocks of eight warps: with
+  // four, each item after the first ones is slower, the more of them the
+  // slower (us, four and eight warps: 256^3, 256 columns, 768 radii, batch 4
+  // 5460 and 4906, batch 8 11305 and 9768, 64 columns, 1024 radii 1973 and
+  // 1705; 4 x 192^3, 128 columns 2061 and 1832, 32 columns of 184 slabs 592 and
+  // 555).  Two items, or few blocks: 2 x 192^3 1854 and 1893, 4 x 64^2 x 160 234
+  // and 254; one: 256^3 1263 and 1290, 160^3 682 and 717; one chunk of columns:
+  // 128^3 303 and 322, 8 x 96^3 1207 and 1218.
+  const bool big = CH == 2 && batch > 2 && a1t_blocks<8>(A) * batch >= 4096;
+  const int64_t gx = big ? a1t_blocks<8>(A) : a1t_blocks<4>(A);
+  if (gx > 0x7fffffff || batch > 65535) return SRT_ERR_ARG;
   dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
-  if (CH == 2)
-    SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_tile<W, 2>, grid, kNW * 32, st, A, w, x, (int)ldx, bsx,
-                            y, (int)ldy, bsy, ncols));
-  else
-    SRT_CUDA_TRY(srt_launch(3 * kSMs, k_a1t_tile<W, 1>, grid, kNW * 32, st, A, w, x, (int)ldx, bsx,
-                            y, (int)ldy, bsy, ncols));
+#define SRT_A1T(K, NW)                                                                            \
+  SRT_CUDA_TRY(srt_launch(3 * kSMs, K, grid, NW * 32, st, A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, \
+                          ncols))
+  if (A.mode && ncols <= 64) {
+    if (ncols <= 16 && A.mode == 2)  // 8 groups: one to each of the 8 passes
+      SRT_A1T((k_a1t_split<W, 1, 4>), 4);
+    else if (ncols <= 32)
+      SRT_A1T((k_a1t_split<W, 1, 8>), 4);
+    else
+      SRT_A1T((k_a1t_split<W, 1, 16>), 4);
+  } else if (big) {
+    SRT_A1T((k_a1t_tile<W, 2, 8>), 8);
+  } else if (CH == 2) {
+    SRT_A1T((k_a1t_tile<W, 2, 4>), 4);
+  } else {
+    SRT_A1T((k_a1t_tile<W, 1, 4>), 4);
+  }
+#undef SRT_A1T
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }
@@ -590,14 +604,13 @@ int srt_a1tiles_apply(const srt_plan_s* plan, int g0, int g1, const float* x, in
   A.xrows = srt_checked_rows((int64_t)g.n_phi * g.n_ell);
   // tiles (ta, tb), ta in [g0, g1): blocks of 2 x 2 tiles (4 x 4 pixels)
   // walked in 16 x 16 tile (32 x 32 pixel) super-tiles where they fit, so
-  // the rows gathered at any time belong to a compact patch (with
-  // blocks of 4 x 2 tiles 1.457 ms at 256^3, against 1.483 with 32 x 32
-  // tiles and 1.469 with none; blocks of 4 x 1 tiles 1.276, of 2 x 2 1.272)
+  // the rows gathered at any time belong to a compact patch (256^3: blocks of
+  // 2 x 2 tiles 1.263 ms, of 4 x 1 1.266; 32 x 32 tiles 1.265, none 1.256, but
+  // none 1.703 against 1.670 with 1024 radii; blocks of 4 x 2 tiles 1.290)
   A.g0 = g0;
   A.g1 = g1;
   A.G = g1 - g0;
   A.R = t.ntx;
-  A.TG = 2;
   A.S = (A.G % 16 == 0 && A.R % 16 == 0) ? 16 : 0;
   if (g.weight_dtype == SRT_BF16) {
     const uint2* w = reinterpret_cast<const uint2*>(t.aw16);

@@ -203,8 +203,8 @@ struct SrtRot {
 // r0 <= r < r0 + rows (rows < 0: to A's end) and n < ncols.  With G > 0 the
 // launch's rows (G groups of R) are visited chunk-major across groups, a
 // block owning TG groups (1, 2, 4 or 8) x 8/TG consecutive rows of each.
-// With S > 0 (dividing G and R) the blocks walk S x S super-tiles of the
-// G x R row grid instead of chunk-major bands.  ldn > 0 (A1 with rot.mode
+// With S > 0 (S or S / 2 dividing G and R) the blocks walk S x S super-tiles
+// of the G x R row grid (or S / 2) instead of chunk-major bands.  ldn > 0 (A1 with rot.mode
 // 1, G = n_phi, R = n_ell, ncols = mz, batch items b): y is Y1', the
 // output of the reshape P1, y[(l ncols + k) ldn + b G + j] for row (j, l).
 int srt_spmm(const SrtCsr& A, int weight_dtype, const float* x, int64_t ldx, int64_t bsx, float* y,

@@ -153,7 +153,7 @@ constexpr int kBlockWarps = GL > 8 ? 8 : 4;
 // shared memory, 128 slabs at a time, and are written as Y1'[(l, k)][b G +
 // j], row stride ldn, 16 bytes (4 sensor columns) per radius and slab.
 template <typename V, int VW, int CH, int GL, int MODE, bool TR, int U>
-__global__ void __launch_bounds__(kBlockWarps<GL> * 32)
+__global__ void __launch_bounds__(kBlockWarps<GL> * 32, MODE == 2 && U == 1 ? 6 : 0)
     k_rows(int rows, int r0, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
            const V* __restrict__ val, const float* __restrict__ x, int64_t ldx, int64_t bsx,
            float* __restrict__ y, int64_t ldy, int64_t bsy, int ncols, int G, int R, int TG, int S,
@@ -410,8 +410,11 @@ int launch_width(const SrtCsr& A, const V* val, const Rows& W, const float* x, i
   if constexpr (VW == 4)
     if (m <= 24) SRT_ROWS(3, 8);
   if (m <= 32) SRT_ROWS(2, 16);
+  // (A1^T rows in two chunks of a whole warp, unless few: 192^3 by symmetry
+  // 1368 -> 1195 us, 160^3 936 -> 881, 191^2 x 192 1370 -> 1226; A1 and A2 rows are
+  // faster in three chunks of a half warp, A1 at 192^3 by 3%)
   if constexpr (VW == 4)
-    if (m <= 48) SRT_ROWS(3, 16);
+    if (m <= 48 && (U == 4 || parts > 1 || !(MODE == 2 || (MODE == 0 && W.S > 0)))) SRT_ROWS(3, 16);
   if constexpr (VW != 4) {
     if (m > 96) SRT_ROWS(4, 32);
     if (m > 64) SRT_ROWS(3, 32);
@@ -444,6 +447,14 @@ int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t
   if constexpr (MODE != 1 && MODE != 2)
     if (lanes == 4 && vecs > 64)
       return launch_width<V, 4, MODE, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+  // A1^T rows by symmetry of more than 192 slabs walking super-tiles: one
+  // gather at a time at 40 registers, 48 warps per SM, which suits that walk's
+  // reuse in L2 better than two at 60 (256^3, 768 radii 1668 -> 1607 us, batch 4
+  // 6473 -> 6166, 224^3 1727 -> 1648; with 1024 radii 2121 -> 2174; without
+  // super-tiles 240^3 1922 -> 2063)
+  if constexpr (MODE == 2)
+    if (lanes == 4 && vecs > 48 && vecs <= 64 && !few && W.S > 0)
+      return launch_as<V, 4, 2, 32, 2, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
 #define SRT_WIDTH(VW)                                                                          \
   return few ? launch_width<V, VW, MODE, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, \
                                             st)                                               \
@@ -485,6 +496,7 @@ int srt_spmm(const SrtCsr& A, int wdt, const float* x, int64_t ldx, int64_t bsx,
   }
   if (G > 0 && (int64_t)G * R != rows) G = 0;
   if (TG != 1 && TG != 2 && TG != 4 && TG != 8) TG = 1;
+  if (S > 0 && (G % S || R % S)) S /= 2;  // (160^3 891 -> 881 us, 224^3 1730 -> 1693)
   if (G <= 0 || S <= 0 || G % S || R % S || S % TG) S = 0;
   // gathered operand: A's columns, or for A1^T from the stored quarter
   // (mode 2) the rows (j, l) of every sensor column

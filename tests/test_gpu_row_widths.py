@@ -89,3 +89,28 @@ def test_a1t_of_large_batches(srt, orc, ms, mz, batch, form):
     a = plan.adjoint(y)
     for b in range(batch):
         assert torch.equal(a[b], plan.adjoint(y[b].contiguous()))
+
+
+def _batches_equal_single_items(plan, fn, shape, batches, seed):
+    import torch
+    x = torch.randn((max(batches), *shape), generator=torch.Generator(device="cuda").manual_seed(seed), device="cuda")
+    one = [fn(x[b].contiguous()).clone() for b in range(max(batches))]
+    for n in batches:
+        if n > 1:
+            y = fn(x[:n].contiguous())
+            assert all(torch.equal(y[b], one[b]) for b in range(n)), n
+    return one
+
+
+@pytest.mark.parametrize("mz", [8, 32, 33, 34, 64, 66, 100, 101, 128, 132, 160, 192, 200, 202, 256, 264])
+@pytest.mark.parametrize("ms", [127, 128])
+@pytest.mark.parametrize("form", [dict(), dict(a1_full=True), dict(weight_dtype="bf16")])
+def test_pixel_rows_bitwise_over_batches(srt, orc, mz, ms, form):
+    """A1^T row by row at 128 x 128 pixels: one volume counts as few rows, five
+    as many (two from 132 slabs on), so the same sums run with four, two and
+    one gathers in flight, in half warps and whole ones, over super-tiles
+    (128) and bands (127)."""
+    g, _ = geom_pair(orc, ms=ms, mz=mz, dxy=0.2, dz=0.2, radius=20.0, n_phi=8, n_zs=3, n_ell=14, rowwise=True,
+                     **form)
+    plan = srt.Plan(g)
+    _batches_equal_single_items(plan, plan.adjoint, g.p_shape, (1, 2, 5), 7)

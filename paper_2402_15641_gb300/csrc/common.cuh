@@ -401,6 +401,10 @@ __host__ __device__ inline uint16_t srt_f64_to_bf16(double x) {
   return (uint16_t)((sign << 15) | q);
 }
 
+// Is entry e before its row's end e1?  Entries are numbered up to 2^31 - 1
+// and a batch asks past its row's end, so e is formed and compared unsigned.
+__host__ __device__ inline bool srt_in_row(uint32_t e, uint32_t e1) { return e < e1; }
+
 // Loads of a kernel's operand (see srt_in_order): plain global loads, not
 // read-only ones, and volatile, so that they stay behind the wait.
 //

@@ -218,20 +218,21 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32, MODE == 2 && U == 1 ? 6 
   for (int s = 0; s < (MODE == 2 ? 4 : 1); ++s) {
     if (MODE == 2) sr = rot_pixel(row, 4 - s, ms, magic);
     const int off = MODE == 2 ? s * q * n_ell : 0;
-    const int e0 = rowptr[sr];
-    const int e1 = mine ? rowptr[sr + (MODE == 3 ? ms : MODE == 4 ? q : 1)] : e0;
+    // (unsigned: a batch asks past its row's end, where 2^31 may be passed)
+    const uint32_t e0 = rowptr[sr];
+    const uint32_t e1 = mine ? rowptr[sr + (MODE == 3 ? ms : MODE == 4 ? q : 1)] : e0;
     // batches run in step over the warp's rows (an exhausted row idles); the
     // next batch's entries are requested before this one's gathers
-    const int len = NR > 1 ? (int)__reduce_max_sync(FULL, (unsigned)(e1 - e0)) : e1 - e0;
+    const int len = NR > 1 ? (int)__reduce_max_sync(FULL, e1 - e0) : (int)(e1 - e0);
     constexpr int KE = EB / GL;
     // (short rows of single columns have too few gathers to cover the request)
     constexpr bool PF = !SH && !(VW == 1 && U == 4);
     int nc[KE];
     V nv[KE];
-    auto ask = [&](int eb) {
+    auto ask = [&](uint32_t eb) {
 #pragma unroll
       for (int k = 0; k < KE; ++k)
-        if (eb + sl + k * GL < e1) {
+        if (srt_in_row(eb + sl + k * GL, e1)) {
           nc[k] = col[eb + sl + k * GL];
           nv[k] = val[eb + sl + k * GL];
         }
@@ -239,17 +240,17 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32, MODE == 2 && U == 1 ? 6 
     if (PF) ask(e0);
 #pragma unroll 1
     for (int b = 0; b < len; b += EB) {
-      const int eb = e0 + b;
+      const uint32_t eb = e0 + b;
       if constexpr (SH) {
         int c = 0;
         float v = 0.f;
-        if (eb + lane < e1) {
+        if (srt_in_row(eb + lane, e1)) {
           c = col[eb + lane];
           c = remap(c, off);
           SRT_CHECK_GATHER(0, c, xrows, g_viol);
           v = wval<V>(val[eb + lane]);
         }
-        const int cnt = min(32, e1 - eb);
+        const int cnt = min(32, (int)(e1 - eb));
 #pragma unroll 1
         for (int i = 0; i < cnt; ++i) {
           const int ci = __shfl_sync(FULL, c, i);
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32, MODE == 2 && U == 1 ? 6 
       if (!PF) ask(eb);
 #pragma unroll
       for (int k = 0; k < KE; ++k)
-        if (eb + sl + k * GL < e1) {
+        if (srt_in_row(eb + sl + k * GL, e1)) {
           int c = nc[k];
           c = remap(c, off);
           SRT_CHECK_GATHER(0, c, xrows, g_viol);
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kBlockWarps<GL> * 32, MODE == 2 && U == 1 ? 6 
         }
       if (PF) ask(eb + EB);
       __syncwarp();
-      const int cnt = min(EB, e1 - eb);
+      const int cnt = min(EB, (int)(e1 - eb));
       int i = 0;
 #pragma unroll 1
       for (; i + U <= cnt; i += U) {

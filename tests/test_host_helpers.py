@@ -69,6 +69,22 @@ def test_bf16_rounding(run):
     assert [int(g) for g in got] == [_bf16_code(float(x)) for x in xs]
 
 
+def test_entry_of_a_row_at_the_int32_limit(run):
+    """The last rows of an operator of nearly 2^31 entries: a batch asks for
+    entries past the end of its row (its own last batch, the one after, or
+    another, longer row's of the same warp), whose number does not fit 32 bits."""
+    top = 2 ** 31 - 1
+    cases = [(e0, e1, i) for e0, e1 in ((0, 0), (0, 5), (top - 9, top), (top - 2000, top - 1990), (top, top))
+             for i in (0, 4, 5, 8, 9, 10, 15, 16, 31, 48, 2100, 100000)]
+    got = run([f"ent {e0} {e1} {i}" for e0, e1, i in cases])
+    assert [int(g) for g in got] == [int(e0 + i < e1) for e0, e1, i in cases]  # exact integers here
+    src = open(os.path.join(ROOT, "paper_2402_15641_gb300", "csrc", "spmm.cu")).read()
+    body = src[src.index("k_rows(int rows"):src.index("// Columns of one launch")]
+    assert "< e1" not in body  # every batch asks srt_in_row, with unsigned numbers
+    for name in ("e0", "e1", "eb"):
+        assert f"const uint32_t {name} =" in body and f"int {name}" not in body
+
+
 def _arc_cases(rng, n):
     cases = []
     for _ in range(n):

@@ -6,7 +6,8 @@
 // row fetched per entry).  A circle crossing a pixel usually crosses its
 // neighbour too, so a warp owns a 2 x 2 tile of pixels (rows of A1^T) and
 // walks the union of its rows' gathered rows: one record per gathered row,
-// with four weights (zero where a pixel does not use it).  At 256^3 a record
+// with four weights (zero, and skipped, where a pixel does not use it, so an
+// infinite or NaN sample reaches only the pixels that do).  At 256^3 a record
 // serves 2.0 entries on average.  (The same idea for A1 itself, 4
 // consecutive radii of one column per warp, measured slower than the CSR
 // row kernel: there the rows of a block already share their gathered pixels
@@ -227,12 +228,15 @@ __device__ __forceinline__ void a1t_pass(const A1Args& A, const W* __restrict__ 
     const float* xr = x0 + (int64_t)row_of(__ldg(A.key + e)) * ldx;
     float w[4];
     rec_w<W>(wt + e, w);
+    float4 v[CH];
 #pragma unroll
     for (int c = 0; c < CH; ++c)
-      if (in[c]) {
-        const float4 xv = srt_ld_keep(xr + c * 128);
+      if (in[c]) v[c] = srt_ld_keep(xr + c * 128);
 #pragma unroll
-        for (int sg = 0; sg < 4; ++sg) fma4(acc[sym_slot(PS, PM, sg)][c], w[sg], xv);
+    for (int sg = 0; sg < 4; ++sg)
+      if (w[sg] != 0.f) {
+#pragma unroll
+        for (int c = 0; c < CH; ++c) fma4(acc[sym_slot(PS, PM, sg)][c], w[sg], v[c]);
       }
   }
 }

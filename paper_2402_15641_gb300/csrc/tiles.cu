@@ -32,7 +32,9 @@
 // 0 <= c + delta < mz; adjoint: 0 <= c + gamma < n_zs) are one contiguous
 // range.  Each output row therefore sums its entries in the order of the
 // taps kernel: ascending (offset, l) in the forward, ascending (h, m) (the
-// CSR order of A2^T) in the adjoint; the padded zero weights add +0.
+// CSR order of A2^T) in the adjoint.  A zero weight, which stands for a row
+// that does not use the gathered row, is skipped, so an infinite or NaN
+// sample reaches the rows that hold an entry for it and no others.
 //
 // The reshape that follows each product in Algorithms 1 and 2 (P2 after A2,
 // P1^-1 after A2^T) can be folded into the product's epilogue (TR): the
@@ -228,12 +230,15 @@ __global__ void __launch_bounds__(TR ? 256 : 128, TR ? 2 : 4)
       float w[4];
       tile_w<W>(wt + e, w);
       const float* xr = x0 + (int64_t)o * ldx;
+      float4 v[CH];
 #pragma unroll
       for (int q = 0; q < CH; ++q)
-        if (in[q]) {
-          const float4 xv = srt_ld_keep(xr + q * 128);
+        if (in[q]) v[q] = srt_ld_keep(xr + q * 128);
 #pragma unroll
-          for (int s = 0; s < 4; ++s) fma4(acc[s][q], w[s], xv);
+      for (int s = 0; s < 4; ++s)
+        if (w[s] != 0.f) {
+#pragma unroll
+          for (int q = 0; q < CH; ++q) fma4(acc[s][q], w[s], v[q]);
         }
     }
   }

@@ -143,9 +143,10 @@ constexpr int kBlockWarps = GL > 8 ? 8 : 4;
 // columns a whole warp to a row leaves lanes idle and spends the same loop
 // on fewer columns; with GL lanes to a row (measured, one box, FP32 entries,
 // a warp to a row before): 8 x 64^3 446 -> 212 us, 128^3 416 -> 340, 192^3
-// 1180 -> 1072.  U gathers are requested before their FMAs: two cost no
-// registers' worth of residency (32, 64 warps per SM) and gain 4% at 128^3;
-// four cost 6% at 256^3 but win where the launch cannot fill the GPU.
+// 1180 -> 1072.  U gathers are requested before their FMAs: two gain 4% at
+// 128^3, at 54 registers and 32 warps per SM in the kernel of 256 columns (48 to
+// 72 registers in the others); four, at 72 to 99 registers and 16 to 24 warps,
+// cost 6% at 256^3 but win where the launch cannot fill the GPU.
 // A row's entries are summed in the same order in every variant.
 //
 // TR (MODE 1, GL = 32, blocks of 4 sensor columns x 2 radii, G = n_phi, R =
@@ -395,36 +396,39 @@ int launch_width(const SrtCsr& A, const V* val, const Rows& W, const float* x, i
   const int n = (ncols + VW - 1) / VW;  // vectors of a row
   // wide rows stored as they are: each entry's reuse over 512 columns wins
   // over more warps (at 1024 columns 10.6 against 11.1 ms for A2 of 256^3 as CSR)
-  if constexpr (MODE != 1 && MODE != 2 && VW == 4 && U == 1) {
+  if constexpr (U == 1) {
     if (n > 96) SRT_ROWS(4, 32);
     SRT_ROWS(3, 32);
+  } else {
+    // rows wider than a part in equal parts (64 float4 vectors, 128 narrower
+    // ones: what a warp covers in two chunks or in up to four light ones);
+    // then the narrowest group that covers a part
+    constexpr int P = VW == 4 ? 64 : 128;
+    const int parts = (n + P - 1) / P, m = (n + parts - 1) / parts;
+    // Too few rows for 32 warps per SM even with a half warp to a row: the
+    // time is one row's chain of gathers, and packing more rows into a warp
+    // only lengthens it to the longest of them (A1 at 32^3, 8 vectors: 13.5 us
+    // with a half warp to a row, 17.9 with four lanes; at 64^3, 44.5 against 41.2
+    // the other way round, half warps losing).
+    if (m <= 8 && (int64_t)W.rows * batch * parts <= (int64_t)2 * 32 * kSMs) SRT_ROWS(2, 16);
+    if (m <= 8) SRT_ROWS(2, 4);
+    if (m <= 16) SRT_ROWS(2, 8);
+    if constexpr (VW == 4)
+      if (m <= 24) SRT_ROWS(3, 8);
+    if (m <= 32) SRT_ROWS(2, 16);
+    // (A1^T rows in two chunks of a whole warp, unless few: 192^3 by symmetry
+    // 1368 -> 1195 us, 160^3 936 -> 881, 191^2 x 192 1370 -> 1226; A1 and A2 rows are
+    // faster in three chunks of a half warp, A1 at 192^3 by 3%)
+    if constexpr (VW == 4)
+      if (m <= 48 && (U == 4 || parts > 1 || !(MODE == 2 || (MODE == 0 && W.S > 0)))) SRT_ROWS(3, 16);
+    // (parts of 64 vectors instead: A2 of 191 columns at 126 slabs 959 us, 707 so;
+    // A1^T of 187 slabs 1307, 1023)
+    if constexpr (VW != 4) {
+      if (m > 96) SRT_ROWS(4, 32);
+      if (m > 64) SRT_ROWS(3, 32);
+    }
+    SRT_ROWS(2, 32);
   }
-  // rows wider than a part in equal parts (64 float4 vectors, 128 narrower
-  // ones: what a warp covers in two chunks or in up to four light ones);
-  // then the narrowest group that covers a part
-  constexpr int P = VW == 4 ? 64 : 128;
-  const int parts = (n + P - 1) / P, m = (n + parts - 1) / parts;
-  // Too few rows for 32 warps per SM even with a half warp to a row: the
-  // time is one row's chain of gathers, and packing more rows into a warp
-  // only lengthens it to the longest of them (A1 at 32^3, 8 vectors: 13.5 us
-  // with a half warp to a row, 17.9 with four lanes; at 64^3, 44.5 against 41.2
-  // the other way round, half warps losing).
-  if (m <= 8 && (int64_t)W.rows * batch * parts <= (int64_t)2 * 32 * kSMs) SRT_ROWS(2, 16);
-  if (m <= 8) SRT_ROWS(2, 4);
-  if (m <= 16) SRT_ROWS(2, 8);
-  if constexpr (VW == 4)
-    if (m <= 24) SRT_ROWS(3, 8);
-  if (m <= 32) SRT_ROWS(2, 16);
-  // (A1^T rows in two chunks of a whole warp, unless few: 192^3 by symmetry
-  // 1368 -> 1195 us, 160^3 936 -> 881, 191^2 x 192 1370 -> 1226; A1 and A2 rows are
-  // faster in three chunks of a half warp, A1 at 192^3 by 3%)
-  if constexpr (VW == 4)
-    if (m <= 48 && (U == 4 || parts > 1 || !(MODE == 2 || (MODE == 0 && W.S > 0)))) SRT_ROWS(3, 16);
-  if constexpr (VW != 4) {
-    if (m > 96) SRT_ROWS(4, 32);
-    if (m > 64) SRT_ROWS(3, 32);
-  }
-  SRT_ROWS(2, 32);
 #undef SRT_ROWS
 }
 
@@ -440,10 +444,11 @@ int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t
   }
   const int64_t any = ncols | ldx | ldy | bsx | bsy;
   const uintptr_t at = (uintptr_t)x | (uintptr_t)y;
-  // Four gathers in flight per row where the rows do not keep the SMs full
-  // for more than two rounds of 64 warps (75 x 75 x 53, 18090 rows: A1 44.8
-  // -> 35.8 us, A1^T 47.1 -> 36.9; 32^3: 18.6 -> 13.5), two otherwise (96^3,
-  // 24576 warps of four rows: 207 us with four, 188 with two).
+  // Four gathers in flight per row up to 128 warps' worth of rows per SM, five
+  // to eight times what the registers of the variants leave room for at once
+  // (75 x 75 x 53, 18090 rows: A1 44.8 -> 35.8 us, A1^T 47.1 -> 36.9; 32^3: 18.6 ->
+  // 13.5), two above (96^3, 24576 warps of four rows: 207 us with four, 188 with
+  // two).
   const int lanes = any % 4 == 0 && at % 16 == 0 ? 4 : any % 2 == 0 && at % 8 == 0 ? 2 : 1;
   const int64_t vecs = ((int64_t)ncols + lanes - 1) / lanes;
   const int64_t per_warp = vecs > 32 ? 1 : vecs > 16 ? 2 : 4;
@@ -467,7 +472,14 @@ int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t
                                             st)
   if (lanes == 4) SRT_WIDTH(4);
   if (lanes == 2) SRT_WIDTH(2);
-  SRT_WIDTH(1);
+  // Single columns of A1^T and of the taps: four gathers, many rows or few (us,
+  // four and two: A2 of 191 columns at 126 slabs 707 and 799, of 171 at 187 2247
+  // and 2560; A1^T of 187 slabs 1023 and 1072); pairs of columns gain nothing
+  // there (A2 of 190 columns at 127 slabs 498 and 492).
+  if constexpr (MODE >= 2)
+    return launch_width<V, 1, MODE, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+  else
+    SRT_WIDTH(1);
 #undef SRT_WIDTH
 }
 

@@ -1,8 +1,11 @@
-"""The row products at every width class of their dispatch: vectors of 4, 2
-and 1 columns, 4 to 32 lanes to a row, one to three chunks, rows split over
-blocks, few rows (four gathers in flight) and many (two), against the FP64
-oracle on seeded samples.  The bound is that of FP32 sums of a row's entries
-(at most a few hundred), 1e-5 relative, as in the parity tests."""
+"""The row products over the width classes of their dispatch: vectors of 4, 2
+and 1 columns, 4 to 32 lanes to a row, two to four chunks, rows split over
+blocks, few rows (four gathers in flight) and many (two, or one).
+
+Against the FP64 oracle on seeded samples, with the bound of FP32 sums of a
+row's entries (at most a few hundred), 1e-5 relative, as in the parity tests;
+and bitwise between batch sizes: every variant sums a row in the same order, so
+an item's result does not depend on the variant that its batch selects."""
 import numpy as np
 import pytest
 
@@ -114,3 +117,37 @@ def test_pixel_rows_bitwise_over_batches(srt, orc, mz, ms, form):
                      **form)
     plan = srt.Plan(g)
     _batches_equal_single_items(plan, plan.adjoint, g.p_shape, (1, 2, 5), 7)
+
+
+@pytest.mark.parametrize("mz", [8, 16, 18, 21, 32, 33, 36, 48, 62, 64, 66, 80, 96, 100, 101, 128, 130, 132, 160,
+                                192, 200, 201, 256, 258, 264, 300])
+@pytest.mark.parametrize("form", [dict(), dict(a1_full=True), dict(weight_dtype="bf16")])
+def test_a1_rows_bitwise_over_batches(srt, orc, mz, form):
+    """A1 with 19264 rows an item, more than half a warp each fills the GPU with:
+    one item counts as few rows, two as many where a row has more than 32
+    vectors, five as many at every width."""
+    g, _ = geom_pair(orc, ms=10, mz=mz, dxy=0.4, dz=0.1, radius=6.0, n_phi=64, n_zs=2, n_ell=301, **form)
+    plan = srt.Plan(g)
+    _batches_equal_single_items(plan, plan.forward, g.f_shape, (1, 2, 5), 9)
+
+
+@pytest.mark.parametrize("n_phi", [3, 5, 8, 12, 16, 20, 24, 30, 33, 40, 48, 57, 64, 66, 72, 90, 101, 130])
+@pytest.mark.parametrize("form", [dict(rowwise=True), dict(csr_only=True, rowwise=True),
+                                  dict(rowwise=True, weight_dtype="bf16")])
+def test_shell_rows_bitwise_over_batches(srt, orc, n_phi, form):
+    """A2 and A2^T row by row, from the taps and as CSR, with 20480 rows: the
+    dense width is the batch's columns, so one, two, three and eight items run in
+    different width classes."""
+    g, _ = geom_pair(orc, ms=6, mz=64, dxy=0.4, dz=0.1, radius=6.0, n_phi=n_phi, n_zs=64, n_ell=320, **form)
+    plan = srt.Plan(g)
+    _batches_equal_single_items(plan, plan.forward, g.f_shape, (1, 2, 3, 8), 11)
+    _batches_equal_single_items(plan, plan.adjoint, g.p_shape, (1, 2, 3, 8), 12)
+
+
+@pytest.mark.parametrize("n_ell,batch", [(38, 1), (39, 1), (304, 1), (305, 1), (304, 2), (38, 8)])
+def test_edges_of_the_row_rules(srt, orc, n_ell, batch):
+    """Just below and above the row counts at which the variants change (9728:
+    four lanes a row; 77824 rows of four to a warp, 19456 of one: two gathers)."""
+    for mz, n_phi in ((8, 256), (64, 256), (136, 64)):
+        sz = dict(ms=8, mz=mz, dxy=0.4, dz=0.05, radius=6.0, n_phi=n_phi, n_zs=2, n_ell=n_ell)
+        _sample_check(srt, orc, sz, dict(), batch, 60, 10)

@@ -79,14 +79,16 @@ def test_adjoint_group_passes(srt, orc, mz, form):
         assert rel_l2(a[b], want) <= (5e-3 if bf16 else 1e-5)
 
 
-@pytest.mark.parametrize("ms,mz,batch", [(128, 132, 8), (130, 260, 8), (134, 160, 8), (192, 136, 4)])
+@pytest.mark.parametrize("ms,mz,n_phi,batch", [(128, 132, 72, 8), (130, 260, 16, 8), (134, 160, 16, 8),
+                                                (72, 136, 16, 8)])
 @pytest.mark.parametrize("form", [dict(), dict(a1_full=True), dict(weight_dtype="bf16")])
-def test_a1t_of_large_batches(srt, orc, ms, mz, batch, form):
-    """A1^T of a large batch of more than 128 slabs runs in blocks of 4 x 2
-    tiles, of one volume in 2 x 2: bitwise the same for every item, with tile
-    counts that are and are not whole blocks and super-tiles."""
+def test_a1t_of_large_batches(srt, orc, ms, mz, n_phi, batch, form):
+    """A1^T of more than 128 slabs runs in blocks of 4 x 2 tiles where a batch
+    fills many of them (4096, or 1024 with at most 64 columns), one of these
+    volumes in 2 x 2: bitwise the same for every item, with tile counts that are
+    and are not whole blocks and super-tiles."""
     import torch
-    g, _ = geom_pair(orc, ms=ms, mz=mz, dxy=0.4, dz=0.3, radius=0.4 * ms, n_phi=16, n_zs=5, n_ell=24, **form)
+    g, _ = geom_pair(orc, ms=ms, mz=mz, dxy=0.4, dz=0.3, radius=0.4 * ms, n_phi=n_phi, n_zs=5, n_ell=24, **form)
     plan = srt.Plan(g)
     y = torch.randn((batch, *g.p_shape), generator=torch.Generator(device="cuda").manual_seed(17), device="cuda")
     a = plan.adjoint(y)

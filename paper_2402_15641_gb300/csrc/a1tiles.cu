@@ -48,10 +48,11 @@ __device__ unsigned long long g_viol;  // gathered rows outside their operand
 #endif
 
 // Records per group of the main loop; two groups alternate, as in tiles.cu.
-// The loop is bound by the L1 data pipe and the gathers' latency; blocks of
-// four warps at 128 registers with the FMAs of a record under the test that
-// the slot's weight is not zero (see tiles.cu) take A1^T from 1.391 to 1.265
-// ms at 256^3, and groups of five where 128 columns leave the registers free
+// At 256^3 the L1 data pipe is 75% busy; what holds the rest of the time was
+// not found (eight copies of the loop share 128 registers and reload 120 bytes
+// of spills).  Blocks of four warps at 128 registers with the FMAs of a record
+// under the test that the slot's weight is not zero (see tiles.cu) take A1^T
+// from 1.391 to 1.263 ms there, and groups of five where 128 columns leave the registers free
 // from 434 to 297 us at 128^3 (groups of three 346, four 328, six 307).
 template <int CH>
 constexpr int kH = CH == 2 ? 3 : 5;

@@ -303,8 +303,9 @@ int run_adjoint(srt_plan_s* p, const float* in, float* f, int B, float* w0, floa
   if (!hs) mark(p, 1, 3, st);
   // rows (pixels) in blocks of 4 x 2 pixels: a circle crossing a compact
   // tile touches more of its pixels than of a line of 8, so warps share L1;
-  // blocks walk 64 x 64 pixel super-tiles (where the grid divides), so the
-  // rows gathered at any time stay within what L2 holds (2% faster at 256^3)
+  // blocks walk 64 x 64 pixel super-tiles (or 32 x 32, where the grid divides),
+  // so the rows gathered at any time stay within what L2 holds (2% faster at
+  // 256^3)
   // (tiles: 2 x 2 pixel tiles, chunks of whole tile rows)
   const int span = p->a1tiles ? g.ms / 2 : g.ms;
   const int nc = hs ? (span < hs->chunks ? span : hs->chunks) : 1;

@@ -379,10 +379,10 @@ int launch_as(const SrtCsr& A, const V* val, const Rows& W, const float* x, int6
   if (gx > 0x7fffffff || (ncols + wide - 1) / wide > 65535 || batch > 65535) return SRT_ERR_ARG;
   dim3 grid((unsigned)gx, (ncols + wide - 1) / wide, batch);
   const SrtRot& r = W.rot;
-  SRT_CUDA_TRY(srt_launch(12 * kSMs, k_rows<V, VW, CH, GL, MODE, TR, U>, grid, kBlockWarps<GL> * 32, st, W.rows,
-                          W.r0, A.rowptr, A.col, val, x, ldx, bsx, y, ldy, bsy, ncols, W.G, W.R,
-                          W.TG, S, r.ms,
-      r.n_ell, r.q, r.mirror, W.magic, W.xrows, W.ldn));
+  SRT_CUDA_TRY(srt_launch(12 * kSMs, k_rows<V, VW, CH, GL, MODE, TR, U>, grid,
+                          kBlockWarps<GL> * 32, st, W.rows, W.r0, A.rowptr, A.col, val, x, ldx, bsx,
+                          y, ldy, bsy, ncols, W.G, W.R, W.TG, S, r.ms, r.n_ell, r.q, r.mirror,
+                          W.magic, W.xrows, W.ldn));
   SRT_CUDA_TRY(cudaGetLastError());
   return SRT_OK;
 }

@@ -120,10 +120,9 @@ __device__ __forceinline__ void fma4(float2 (&a)[2], float w, const float4& xv) 
   a[1] = __ffma2_rn(ww, make_float2(xv.z, xv.w), a[1]);
 }
 
-// Records per group of the main loop.  The product waits on its gathers (L2
-// latency), so a warp alternates two groups: it requests the next group's
-// gathered rows before the FMAs of the current one, and its gathers stay in
-// flight while it computes.
+// Records per group of the main loop.  A warp alternates two groups: it
+// requests the next group's gathered rows before the FMAs of the current one,
+// so its gathers stay in flight while it computes.
 //
 // What bounds it, at 256 columns: the L1 data pipe, 94% busy (ncu).  A record
 // takes 8 cycles for its gathered row, 4 for its 16 bytes of weights (a

@@ -116,7 +116,7 @@ def test_unfused_when_width_not_multiple_of_4(srt, orc):
 @pytest.mark.parametrize("sz", [GEOMS[0], GEOMS[2], GEOMS[4]])
 @pytest.mark.parametrize("batch", [1, 3])
 def test_fused_p1_with_rowwise_products(srt, orc, sz, batch):
-    """Row-per-warp products (A1 by quarter turns, no register tiles): only
+    """Products row by row (A1 by quarter turns, no register tiles): only
     P1 folds, into A1; the forward makes 3 launches, the adjoint 4."""
     import torch
     plan, sep, g, o = _plans(srt, orc, sz, rowwise=True)

@@ -302,7 +302,7 @@ def test_toeplitz_second_stage(srt, orc, sz, wdt):
     take less memory than A2 and A2^T (the 2 x 2 tile records add some, which
     on grids this small can outweigh what the taps save), and the transforms
     match the CSR plan and the oracle (dense widths 5 and 15 take the
-    row-per-warp scalar kernel)."""
+    row product of single columns)."""
     g, o = geom_pair(orc, weight_dtype=wdt, **sz)
     a = srt.Plan(g)
     b = srt.Plan(g.with_(csr_only=True))
@@ -428,7 +428,7 @@ def test_a1_by_symmetry(srt, orc, sz, form, wdt):
     8-fold form; n_phi % 8 == 0, phi0 = 0, ms even, mz % 4 == 0), else the
     first n_phi/4 under quarter turns.  The full A1 and A1^T it stands for
     (exported) have the pattern of the directly assembled ones and their FP64
-    entries to rounding, and the transforms (tile and row-per-warp kernels)
+    entries to rounding, and the transforms (tile and row products)
     match the fully stored plan and the oracle (odd ms, a phase phi0, rings
     off the slab centres, an odd radius count, two stored columns that are
     both fixed by a mirror, BF16, batch 2)."""
@@ -466,9 +466,9 @@ def test_a1_by_symmetry(srt, orc, sz, form, wdt):
 @pytest.mark.parametrize("batch", [1, 3])
 def test_a1_tiles_equal_rowwise(srt, orc, sz, wdt, batch):
     """With A1 stored for every column, the 2 x 2 pixel A1^T tiles sum every
-    pixel's entries in the CSR order of A1^T (ascending (j, l)) and add only
+    pixel's entries in the CSR order of A1^T (ascending (j, l)) and skip the
     zeros besides, and the A2 tiles those of the taps: forward and adjoint
-    equal the row-per-warp kernels bitwise (after +0.0, which equates the
+    equal the row products bitwise (after +0.0, which equates the
     signs of zero sums)."""
     import torch
     g, _ = geom_pair(orc, weight_dtype=wdt, a1_full=True, **sz)
@@ -542,8 +542,8 @@ TILE_GEOMS = [dict(I.sizes("srt32")), dict(I.sizes("srt16fd")),
 @pytest.mark.parametrize("wdt", ["fp32", "bf16"])
 @pytest.mark.parametrize("batch", [1, 3])
 def test_tiles_equal_rowwise_taps(srt, orc, sz, wdt, batch):
-    """The 2 x 2 row tiles sum every row in the order of the row-per-warp
-    taps kernel and add only zeros besides, so forward and adjoint agree
+    """The 2 x 2 row tiles sum every row in the order of the taps' row
+    product and skip the zeros besides, so forward and adjoint agree
     bitwise (after +0.0, which equates the signs of zero sums; A1 stored for
     every column in both plans, where its tiles are bitwise the CSR rows
     too); odd ring, slab and radius counts leave half-empty tiles at the

@@ -31,25 +31,33 @@ def _body(s, start):
     raise AssertionError("unbalanced braces")
 
 
-def _kernels():
-    """(file, kernel, operand parameter, body) of every kernel srt_launch starts."""
+def _kernels(early):
+    """(file, kernel, operand parameter, body) of every kernel that waits for
+    the one before (early) or of every other."""
     out = []
     for f in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
         s = _source(f)
-        launched = set(re.findall(r"srt_launch\([^;]*?\b(k_\w+)", s))
         for m in re.finditer(r"__global__[^;{]*?\b(k_\w+)\(([^{;]*?)\)\s*\{", s):
-            if m.group(1) in launched:
+            body = _body(s, m.end() - 1)
+            if ("srt_in_order" in body) == early:
                 operand = re.findall(r"const float\*\s*(?:__restrict__)?\s*(\w+)", m.group(2))
-                out.append((os.path.basename(f), m.group(1), operand, _body(s, m.end() - 1)))
+                out.append((os.path.basename(f), m.group(1), operand, body))
     return out
 
 
 def test_every_early_kernel_is_found():
-    assert {k for _, k, _, _ in _kernels()} == {"k_rows", "k_tile22", "k_a1t_tile", "k_a1t_split",
-                                                "k_transpose", "k_transpose_v4"}
+    early = {k for _, k, _, _ in _kernels(True)}
+    assert early == {"k_rows", "k_tile22", "k_a1t_tile", "k_a1t_split", "k_transpose", "k_transpose_v4"}
+    # the others are launched in order, by <<< >>>, and these never are
+    for f in glob.glob(os.path.join(CSRC, "*.cu")):
+        s = _source(f)
+        plain = set(re.findall(r"\b(k_\w+)(?:<[^;<>]*>)?\s*<<<", s))
+        assert not plain & early, f
+        for name in set(re.findall(r"__global__[^;{]*?\b(k_\w+)\(", s)) - early:
+            assert name in plain, name
 
 
-@pytest.mark.parametrize("file,kernel,operand,body", _kernels(), ids=lambda v: v if isinstance(v, str) and
+@pytest.mark.parametrize("file,kernel,operand,body", _kernels(True), ids=lambda v: v if isinstance(v, str) and
                          len(v) < 20 else "")
 def test_waits_first_and_reads_its_operand_behind_the_wait(file, kernel, operand, body):
     assert body.lstrip().startswith("srt_in_order();")

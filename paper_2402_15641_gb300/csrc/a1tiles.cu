@@ -551,19 +551,20 @@ int launch_a1t(const A1Args& A, const W* w, const float* x, int64_t ldx, int64_t
                int64_t ldy, int64_t bsy, int ncols, int batch, cudaStream_t st) {
   const int CH = ncols > 128 ? 2 : 1;
   // More than 128 slabs, blocks of eight warps where the tiles' lists are short
-  // or the batch is large: with four, each item after the first is slower, the
-  // more of them the slower, and with few sensor columns the first as well (us,
-  // four and eight warps: 256^3, 256 columns, 768 radii, batch 2 2576 and 2488, 4
-  // 5460 and 4902, 8 11305 and 9754; 1024 radii, 64 columns, batch 1 481 and 453, 4
-  // 1973 and 1705; 4 x 192^3, 128 columns 2061 and 1832).  Fewer blocks: 2 x 192^3
-  // 1854 and 1893, 4 x 64^2 x 160 234 and 254; one volume of more columns: 256^3
-  // 1263 and 1290, 160^3 682 and 717, 128 columns of 224^2 x 192 in BF16 707 and
-  // 719; one chunk of slabs: 128^3 303 and 322, 8 x 96^3 1207 and 1218.
-  const int64_t b8 = a1t_blocks<8>(A) * batch;
-  const bool big = CH == 2 && (A.n_phi <= 64 ? b8 >= 1024 : batch > 1 && b8 >= 4096);
+  // or the launch is long: with four, the later parts of a long launch are
+  // slower, and with few sensor columns the first as well (us, four and eight
+  // warps: 256^3, 256 columns, 768 radii, batch 2 2576 and 2488, 4 5460 and 4902, 8
+  // 11305 and 9754; 512^3 11787 and 9832; 384^2 x 256 3968 and 3750; 512^2 x 192
+  // 7523 and 6452; 1024 radii, 64 columns, batch 1 481 and 453, 4 1973 and 1705; 4
+  // x 192^3, 128 columns 2061 and 1832).  Fewer blocks: 2 x 192^3 1854 and 1893, 4 x
+  // 64^2 x 160 234 and 254, 320^2 x 256 2615 and 2668, 256^3 1263 and 1290, 160^3 682
+  // and 717, 128 columns of 224^2 x 192 in BF16 707 and 719; one chunk of slabs:
+  // 128^3 303 and 322, 8 x 96^3 1207 and 1218.
+  const int over = (ncols + 128 * CH - 1) / (128 * CH);
+  const bool big = CH == 2 && a1t_blocks<8>(A) * over * batch >= (A.n_phi <= 64 ? 1024 : 4096);
   const int64_t gx = big ? a1t_blocks<8>(A) : a1t_blocks<4>(A);
   if (gx > 0x7fffffff || batch > 65535) return SRT_ERR_ARG;
-  dim3 grid((unsigned)gx, (ncols + 128 * CH - 1) / (128 * CH), batch);
+  dim3 grid((unsigned)gx, over, batch);
 #define SRT_A1T(K, NW)                                                                            \
   SRT_CUDA_TRY(srt_launch(3 * kSMs, K, grid, NW * 32, st, A, w, x, (int)ldx, bsx, y, (int)ldy, bsy, \
                           ncols))

@@ -465,6 +465,15 @@ int launch(const SrtCsr& A, const V* val, const Rows& W, const float* x, int64_t
   if constexpr (MODE == 2)
     if (lanes == 4 && vecs > 48 && vecs <= 64 && !few && W.S > 0)
       return launch_as<V, 4, 2, 32, 2, 1>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+  // A1 whose part of the volume (256 slabs at most) is larger than L2 waits on
+  // DRAM, and four gathers hide more of it (us, two and four: 512^3 15813 and
+  // 15283, 512^2 x 256 10140 and 9819, 384^2 x 256 5026 and 4956; 320^2 x 256, which
+  // L2 holds, 3238 and 3247, 512^2 x 160 in three chunks 7988 and 8364)
+  if constexpr (MODE == 1) {
+    const int64_t parts = (vecs + 63) / 64, m = (vecs + parts - 1) / parts;
+    if (lanes == 4 && m > 48 && A.cols * 16 * m > (int64_t)128 << 20)
+      return launch_width<V, 4, MODE, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, st);
+  }
 #define SRT_WIDTH(VW)                                                                          \
   return few ? launch_width<V, VW, MODE, 4>(A, val, W, x, ldx, bsx, y, ldy, bsy, ncols, batch, \
                                             st)                                               \
